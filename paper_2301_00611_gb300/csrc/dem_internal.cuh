@@ -249,6 +249,9 @@ constexpr int kShiftMax = 511;
 // scan.cu
 size_t scan_workspace_bytes(long long n);
 void exclusive_scan(const int *in, int *out, long long n, int *workspace, cudaStream_t st);
+// two arrays of n items each by the same launches
+void exclusive_scan2(const int *in0, int *out0, const int *in1, int *out1, long long n,
+                     int *workspace, cudaStream_t st);
 
 // collider.cu
 void launch_bbox(const Bodies &b, long long N, double *partials, int nblk, cudaStream_t st);
