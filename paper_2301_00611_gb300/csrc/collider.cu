@@ -6,22 +6,24 @@
 //   1. bin every sphere into a uniform grid of cell edge >= 2 r_max + 2 dL
 //      (periodic: in the wrapped reference cell, keeping the integer image);
 //   2. counting sort over the Morton codes of the cells (atomics only for the
-//      per-cell counts and slots), then sort each cell's bodies by id, so the
+//      per-cell counts and arrival places), each cell's bodies by id, so the
 //      resulting body order ("slots") is deterministic;
 //   3. permute the body arrays into that order (spatial locality for every
 //      later gather);
-//   4. each body scans the forward half of its 27-cell neighbourhood (so each
-//      pair is met once) and keeps the pairs with |x2 + H c - x1| < r1 + r2 + 2 dL,
-//      tested conservatively in FP32 on wrapped coordinates (count, prefix sum,
-//      emit).  A row is oriented by id, not by slot: body 1 is the sphere with the
-//      smaller id (the canonical id1 < id2 of the interaction container), and the
-//      row is stored in body 1's row range, which is then sorted by the id of
-//      body 2;
-//   5. merge the contact history of the previous table into the new rows by
-//      looking each pair up in the old row range of its body 1 (the potential /
-//      real interaction lifecycle of section 3.1.7);
-//   6. build the per-body "down" lists (rows where the body is the second
-//      sphere), sorted by the id of body 1.
+//   4. each body scans its whole 27-cell neighbourhood and keeps
+//      the partners with |x2 + H c - x1| < r1 + r2 + 2 dL, tested conservatively in FP32
+//      on wrapped coordinates; each body's partners are sorted by id on chip.  A
+//      row is oriented by id, not by slot: body 1 is the sphere with the smaller id
+//      (the canonical id1 < id2 of the interaction container), so a body's partners of
+//      larger id are its rows and those of smaller id its "down" list, both in order;
+//   5. prefix sums of the two counts, then one pass over the rows writes them and
+//      merges the contact history of the previous table by looking each pair up in the
+//      old row range of its body 1 (the potential / real interaction lifecycle of
+//      section 3.1.7);
+//   6. one pass over the down entries finds the row of each.
+// Each pair is met from both sides (twice the distance tests of a forward half shell),
+// which is what makes every list come out complete and sorted without atomics, scattered
+// writes or sorts of the table.
 // So a body's rows, down list first, then its own range, run in increasing order
 // of partner id; the force gather sums them in that order.  With the orientation
 // by id, the FP64 arithmetic of a step depends on the bodies and their contact
@@ -65,8 +67,6 @@ __device__ __forceinline__ const Grid &grid_of(const Grid *__restrict__ grids,
   return grids[multi ? sid[i] : 0];
 }
 
-// Cell key of every body; bodies of a removed sub-scene (grid with no cells) get
-// the sentinel key `dead`, which sorts them behind every live body.
 // Order-preserving map of doubles to unsigned integers (sign bit flipped for
 // positives, all bits for negatives), so that integer atomics give min / max.
 __device__ __forceinline__ unsigned long long ord_key(double x) {
@@ -114,9 +114,13 @@ __global__ void k_bbox_sub(const double4_32a *__restrict__ pos, const int *__res
   }
 }
 
+// Cell key, place among the cell's arrivals and walk record (FP32 position relative to the
+// grid, cell, image) of every body; bodies of a removed sub-scene (grid with no cells) get
+// the sentinel key `dead`, which sorts them behind every live body.  The FP64 work of the
+// cell (floor, products, conversions) is done here once; k_reorder permutes the record.
 __global__ void k_bin(const double4_32a *__restrict__ pos, const int *__restrict__ sid, long long N,
                       const Grid *__restrict__ grids, int multi, uint32_t dead, uint32_t *key,
-                      int *count) {
+                      int *rank, int *count, CellRec raw) {
   long long i = (long long)blockIdx.x * kT + threadIdx.x;
   if (i >= N) return;
   const Grid &g = grid_of(grids, sid, multi, i);
@@ -126,46 +130,45 @@ __global__ void k_bin(const double4_32a *__restrict__ pos, const int *__restrict
     int c[3], img[3];
     cell_of(g, p.x, p.y, p.z, c, img);
     m = (uint32_t)cell_index(g, c[0], c[1], c[2]);
+    const double x[3] = {p.x, p.y, p.z};
+    float f[3];
+    for (int k = 0; k < 3; ++k) {
+      double shift = g.L[k] * img[k];
+      if (g.periodic && g.sheared)   // wrapped position x - H img
+        shift = g.H[3 * k] * img[0] + g.H[3 * k + 1] * img[1] + g.H[3 * k + 2] * img[2];
+      f[k] = g.periodic ? (float)(x[k] - shift) : (float)(x[k] - g.lo[k]);
+    }
+    raw.wpos[i] = make_float4(f[0], f[1], f[2], (float)p.w);
+    raw.info[i] = make_int4(c[0] | (c[1] << 10) | (c[2] << 20), img[0], img[1], img[2]);
   }
   key[i] = m;
-  atomicAdd(&count[m], 1);
+  rank[i] = atomicAdd(&count[m], 1);
 }
 
 __global__ void k_scatter(long long N, const uint32_t *__restrict__ key,
-                          const int *__restrict__ start, int *fill, int *tmp) {
+                          const int *__restrict__ rank, const int *__restrict__ start, int *tmp) {
   long long i = (long long)blockIdx.x * kT + threadIdx.x;
-  if (i >= N) return;
-  uint32_t m = key[i];
-  int p = start[m] + atomicAdd(&fill[m], 1);
-  tmp[p] = (int)i;
+  if (i < N) tmp[start[key[i]] + rank[i]] = (int)i;
 }
 
-// sort the bodies of each cell by id: fixes the order the atomics left open
-__global__ void k_cellsort(const int *__restrict__ count, const int *__restrict__ start,
-                           long long ncell, const int *__restrict__ id, int *tmp) {
-  long long m = (long long)blockIdx.x * kT + threadIdx.x;
-  if (m >= ncell) return;
-  int cnt = count[m];
-  if (cnt < 2) return;
-  int s0 = start[m];
-  for (int a = s0 + 1; a < s0 + cnt; ++a) {
-    int v = tmp[a];
-    int key = id[v];
-    int b = a - 1;
-    while (b >= s0 && id[tmp[b]] > key) {
-      tmp[b + 1] = tmp[b];
-      --b;
-    }
-    tmp[b + 1] = v;
-  }
-}
-
+// Bodies to their slots: cell by cell, by id within a cell (the order the atomics left
+// open).  N: the live bodies (the sentinel cell comes last and is dropped).
 __global__ void k_reorder(Bodies src, Bodies dst, long long N, long long cap,
-                          const int *__restrict__ new_to_old, int *slot_of_id, int has_walls,
-                          int mixed, const int *__restrict__ id_shift) {
-  long long p = (long long)blockIdx.x * kT + threadIdx.x;
-  if (p >= N) return;
-  int o = new_to_old[p];
+                          const int *__restrict__ tmp, const uint32_t *__restrict__ key,
+                          const int *__restrict__ start, CellRec raw,
+                          CellRec cr, int *new_to_old, int *slot_of_id, int has_walls, int mixed,
+                          const int *__restrict__ id_shift) {
+  const long long at = (long long)blockIdx.x * kT + threadIdx.x;
+  if (at >= N) return;
+  const int o = tmp[at];
+  const int oid = src.id[o];
+  const uint32_t m = key[o];
+  const int first = start[m], end = start[m + 1];
+  int p = first;
+  for (int q = first; q < end; ++q) p += src.id[tmp[q]] < oid;
+  new_to_old[p] = o;
+  cr.wpos[p] = raw.wpos[o];
+  cr.info[p] = raw.info[o];
   double4_32a x = src.pos[o];
   dst.pos[p] = x;
   const double4_32a v = src.vel[o], w = src.angvel[o];
@@ -176,8 +179,7 @@ __global__ void k_reorder(Bodies src, Bodies dst, long long N, long long cap,
     dst.vw32[2 * p] = make_float4((float)v.x, (float)v.y, (float)v.z, (float)w.x);
     dst.vw32[2 * p + 1] = make_float4((float)w.y, (float)w.z, 0.0f, 0.0f);
     dst.xref32[p] = make_float4((float)x.x, (float)x.y, (float)x.z, 0.0f);
-    const double4_32a mp = src.mprop[o];
-    dst.mprop32[p] = make_float4((float)mp.x, (float)mp.y, (float)mp.z, (float)mp.w);
+    dst.mprop32[p] = src.mprop32[o];
     dst.ori32[p] = src.ori32[o];   // the mixed path keeps the orientation in FP32
   }
   dst.ori[p] = src.ori[o];
@@ -186,274 +188,353 @@ __global__ void k_reorder(Bodies src, Bodies dst, long long N, long long cap,
   dst.xref[p] = make_double4_32a(x.x, x.y, x.z, 0.0);
   const int q = src.sid[o];
   // ids close up over the ranges of removed sub-scenes
-  const int id = src.id[o] - (id_shift ? id_shift[q] : 0);
+  const int id = oid - (id_shift ? id_shift[q] : 0);
   dst.id[p] = id;
   dst.sid[p] = q;
   dst.mat[p] = src.mat[o];
-  dst.flags[p] = src.flags[o];
-  slot_of_id[id] = (int)p;
-  if (has_walls)
-    for (int w = 0; w < 6; ++w) dst.whist[w * cap + p] = src.whist[w * cap + o];
+  const uint8_t flags = src.flags[o];
+  dst.flags[p] = flags;
+  slot_of_id[id] = p;
+  if (has_walls)   // a wall history is read only while its flag is set
+    for (int w = 0; w < 6; ++w)
+      if (flags & (2 << w)) dst.whist[w * cap + p] = src.whist[w * cap + o];
 }
 
-__global__ void k_cellrec(const double4_32a *__restrict__ pos, const int *__restrict__ sid,
-                          long long N, const Grid *__restrict__ grids, int multi, CellRec cr) {
-  long long i = (long long)blockIdx.x * kT + threadIdx.x;
-  if (i >= N) return;
-  const Grid &g = grid_of(grids, sid, multi, i);
-  const double4_32a p = pos[i];
-  int c[3], img[3];
-  cell_of(g, p.x, p.y, p.z, c, img);
-  double x[3] = {p.x, p.y, p.z};
-  float f[3];
-  for (int k = 0; k < 3; ++k) {
-    double shift = g.L[k] * img[k];
-    if (g.periodic && g.sheared)   // wrapped position x - H img
-      shift = g.H[3 * k] * img[0] + g.H[3 * k + 1] * img[1] + g.H[3 * k + 2] * img[2];
-    f[k] = g.periodic ? (float)(x[k] - shift) : (float)(x[k] - g.lo[k]);
-  }
-  cr.wpos[i] = make_float4(f[0], f[1], f[2], (float)p.w);
-  cr.info[i] = make_int4(c[0] | (c[1] << 10) | (c[2] << 20), img[0], img[1], img[2]);
+// Does the shift of j seen from s leave the range of a packed shift?
+__device__ inline bool shift_overflow(const CellRec &cr, int s, int j, int code) {
+  int w[3];
+  code_wrap(code, w);
+  const int4 a = cr.info[s], b = cr.info[j];
+  return abs(a.y - b.y + w[0]) > kShiftMax || abs(a.z - b.z + w[1]) > kShiftMax ||
+         abs(a.w - b.w + w[2]) > kShiftMax;
 }
 
-__device__ inline void unpack_cell(int v, int c[3]) {
-  c[0] = v & 1023;
-  c[1] = (v >> 10) & 1023;
-  c[2] = (v >> 20) & 1023;
-}
-
-// Candidate counts: cnt_up[body 1] and cnt_down[body 2] of every candidate, body 1
-// being the sphere with the smaller id (both arrays zeroed before).  Count and emit read
-// the partners' records through the read-only path (__ldg): nothing in the walk writes
-// them, and the compiler may then issue those loads ahead of the atomics.
-__global__ void k_count(CellRec cr, const int *__restrict__ sid, const int *__restrict__ id,
-                        long long N, const Grid *__restrict__ grids, int multi,
-                        const int *__restrict__ count, const int *__restrict__ start,
-                        int *cnt_up, int *cnt_down, int *err, CandList cl) {
-  long long sl = (long long)blockIdx.x * kT + threadIdx.x;
-  if (sl >= N) return;
-  const int s = (int)sl;
-  const Grid &g = grid_of(grids, sid, multi, sl);
-  const float4 a = cr.wpos[s];
-  const int4 inf = cr.info[s];
-  const int ids = id[s];
-  int ci[3];
-  unpack_cell(inf.x, ci);
-  bool bad = false;
-  int nc = 0;
-  unsigned *mine = cl.list + (long long)s * kCandKeep;
-  for_half_shell(g, count, start, ci, s, [&](int j, const int w[3]) {
-    if (cand_f32(g, a, __ldg(cr.wpos + j), w, g.slack)) {
-      if (cl.use && nc < kCandKeep)   // slot and the neighbour cell's wrap (code 0..26)
-        mine[nc] = (unsigned)j | ((unsigned)((w[0] + 1) + 3 * (w[1] + 1) + 9 * (w[2] + 1)) << 26);
-      ++nc;
-      const bool fwd = ids < __ldg(id + j);
-      atomicAdd(&cnt_up[fwd ? s : j], 1);
-      atomicAdd(&cnt_down[fwd ? j : s], 1);
-      if (g.periodic) {
-        const int4 ij = __ldg(cr.info + j);
-        bad |= abs(inf.y - ij.y + w[0]) > kShiftMax || abs(inf.z - ij.z + w[1]) > kShiftMax ||
-               abs(inf.w - ij.w + w[2]) > kShiftMax;
-      }
-    }
+// Counts of a body whose partners do not fit a list (k_rows and k_downs walk again for it).
+__device__ inline void count_long(const Grid &g, const CellRec &cr, const int *__restrict__ start,
+                                  const int *__restrict__ id, int s, int *cnt_up, int *cnt_down,
+                                  bool &bad) {
+  int up = 0, down = 0;
+  walk_cells<false>(g, cr.wpos, start, cr.info[s].x, s, [&](int j, int code, float, float) {
+    (id[j] > id[s] ? up : down) += 1;
+    if (g.periodic) bad |= shift_overflow(cr, s, j, code);
   });
-  if (cl.use) cl.n[s] = nc;
+  cnt_up[s] = up;
+  cnt_down[s] = down;
+}
+
+// Partners of every body, by partner id: the down partners (smaller ids), then the rows'.
+//
+// Two shapes of the same search.  A thread per body keeps the hits in a shared-memory
+// column and places them by rank (the count of smaller ids): 111 us for 300k bodies at
+// three rows a body, 605 us for 1M at five (a warp per body 223 us for the 300k; a warp
+// per cell 164 and 777 us).  Its 27 cells in turn are a chain of dependent loads, some
+// 55 us however few the bodies, so smaller scenes take a warp per body, a lane per
+// neighbour cell: 7 us for 1000 bodies, 25 us for 20k, 99 us for 100k (a thread per body 61).
+constexpr int kPT = 128;
+constexpr long long kWarpBodies = 65536;
+
+__global__ void __launch_bounds__(kPT) k_partners(CellRec cr, const int *__restrict__ sid,
+                                                  const int *__restrict__ id, long long N,
+                                                  const Grid *__restrict__ grids, int multi,
+                                                  const int *__restrict__ start, int *cnt_up,
+                                                  int *cnt_down, int *err, CandList cl) {
+  __shared__ unsigned ent[kCandKeep][kPT];
+  __shared__ int ids[kCandKeep][kPT];
+  const int tid = threadIdx.x;
+  const long long sl = (long long)blockIdx.x * kPT + tid;
+  if (sl >= N) return;
+  const int s = (int)sl, me = id[s];
+  const Grid &g = grid_of(grids, sid, multi, sl);
+  bool bad = false;
+  int n = 0;
+  walk_cells<false>(g, cr.wpos, start, cr.info[s].x, s, [&](int j, int code, float, float) {
+    if (n < kCandKeep) ent[n][tid] = (unsigned)j | ((unsigned)code << 26);
+    ++n;
+  });
+  if (n > cl.keep) {
+    count_long(g, cr, start, id, s, cnt_up, cnt_down, bad);
+  } else {
+    for (int k = 0; k < n; ++k) {
+      const unsigned e = ent[k][tid];
+      const int j = (int)(e & 0x3ffffffu);
+      ids[k][tid] = __ldg(id + j);
+      if (g.periodic) bad |= shift_overflow(cr, s, j, (int)(e >> 26));
+    }
+    int down = 0;
+    unsigned *mine = cl.list + (long long)s * kCandKeep;
+    for (int k = 0; k < n; ++k) {
+      const int ik = ids[k][tid];
+      int rank = 0;
+      for (int q = 0; q < n; ++q) rank += ids[q][tid] < ik;
+      mine[rank] = ent[k][tid];
+      down += ik < me;
+    }
+    cnt_down[s] = down;
+    cnt_up[s] = n - down;
+  }
   if (bad) atomicOr(err, kErrShiftRange);
 }
 
-// Row of candidate (s, j) in the row range of its body 1 (smaller id) at a position the
-// atomics pick; w: the wrap of j's neighbour cell as seen from s.
-__device__ inline void emit_row(const CellRec &cr, const Bodies &b, const Table &t, int *ufill,
-                                const Grid &g, const int4 &inf, int s, int ids, int j,
-                                const int w[3]) {
-  int c0 = 0, c1 = 0, c2 = 0;   // cell shift of j seen from s
-  if (g.periodic) {
-    const int4 ij = __ldg(cr.info + j);
-    c0 = inf.y - ij.y + w[0]; c1 = inf.z - ij.z + w[1]; c2 = inf.w - ij.w + w[2];
-  }
-  const int idj = __ldg(b.id + j);
-  const bool fwd = ids < idj;
-  const int g1 = fwd ? s : j, g2 = fwd ? j : s;
-  const int r = t.row_start[g1] + atomicAdd(&ufill[g1], 1);
-  if (r < t.row_start[g1 + 1]) {
-    t.pair[r] = make_int2(g1, g2);
-    t.cpack[r] = fwd ? pack_shift(c0, c1, c2) : pack_shift(-c0, -c1, -c2);   // shift of body 2
-    t.found[r] = fwd ? idj : ids;   // sort key: the id of body 2 (scratch until the merge)
-  }
-}
-
-// Rows of the candidates, each in the row range of its body 1 (smaller id) at a
-// position the atomics pick; k_rowsort then fixes the order.  ufill: zeroed.  A walker
-// whose candidates all fit the count pass's list places them from it; the others walk
-// the cells again with the same test.
-__global__ void k_emit(CellRec cr, Bodies b, long long N, const Grid *__restrict__ grids,
-                       int multi, const int *__restrict__ count, const int *__restrict__ start,
-                       Table t, int *ufill, CandList cl) {
-  long long sl = (long long)blockIdx.x * kT + threadIdx.x;
+__global__ void __launch_bounds__(kT) k_partners_warp(CellRec cr, const int *__restrict__ sid,
+                                                      const int *__restrict__ id, long long N,
+                                                      const Grid *__restrict__ grids, int multi,
+                                                      const int *__restrict__ start, int *cnt_up,
+                                                      int *cnt_down, int *err, CandList cl) {
+  __shared__ unsigned ent[kT / 32][kCandKeep];
+  const unsigned all = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const long long sl = ((long long)blockIdx.x * kT + threadIdx.x) >> 5;
   if (sl >= N) return;
-  const int s = (int)sl;
-  const Grid &g = grid_of(grids, b.sid, multi, sl);
-  const int4 inf = cr.info[s];
-  const int ids = b.id[s];
-  const int nc = cl.use ? cl.n[s] : kCandKeep + 1;
-  if (nc <= kCandKeep) {
-    const unsigned *mine = cl.list + (long long)s * kCandKeep;
-    for (int k = 0; k < nc; ++k) {
-      const unsigned e = mine[k];
-      const int j = (int)(e & 0x3ffffffu), code = (int)(e >> 26);
-      const int w[3] = {code % 3 - 1, (code / 3) % 3 - 1, code / 9 - 1};
-      emit_row(cr, b, t, ufill, g, inf, s, ids, j, w);
-    }
-    return;
-  }
+  unsigned *mine = ent[threadIdx.x >> 5];
+  const int s = (int)sl, me = id[s];
+  const Grid &g = grid_of(grids, sid, multi, sl);
   const float4 a = cr.wpos[s];
-  int ci[3];
-  unpack_cell(inf.x, ci);
-  for_half_shell(g, count, start, ci, s, [&](int j, const int w[3]) {
-    if (cand_f32(g, a, __ldg(cr.wpos + j), w, g.slack)) emit_row(cr, b, t, ufill, g, inf, s, ids, j, w);
+  const int packed = cr.info[s].x;
+  const int ci[3] = {packed & 1023, (packed >> 10) & 1023, (packed >> 20) & 1023};
+  const float reach = cand_reach(g);
+  int first = 0, end = 0, code = kNoWrap;
+  if (lane < kStencil) stencil_cell(g, start, ci, lane, first, end, code);
+  float3 at = make_float3(a.x, a.y, a.z);
+  float sh[3] = {0, 0, 0};
+  if (code != kNoWrap && end > first) {
+    int w[3];
+    code_wrap(code, w);
+    wrap_shift_f32(g, w, sh);
+    const float3 mv = moved_f32(sh, code);
+    at = make_float3(__fadd_rn(a.x, mv.x), __fadd_rn(a.y, mv.y), __fadd_rn(a.z, mv.z));
+  }
+  int n = 0;
+  for (int j = first; __any_sync(all, j < end); ++j) {
+    bool keep = false;
+    if (j < end) {
+      const float4 p = __ldg(cr.wpos + j);
+      float d2, R;
+      keep = cand_f32(at, a.w, placed_f32(p, sh, code), p.w, reach, d2, R) && j != s;
+    }
+    const unsigned m = __ballot_sync(all, keep);
+    const int k = n + __popc(m & ((1u << lane) - 1u));
+    if (keep && k < kCandKeep) mine[k] = (unsigned)j | ((unsigned)code << 26);
+    n += __popc(m);
+  }
+  __syncwarp();
+  bool bad = false;
+  if (n > cl.keep) {
+    if (lane == 0) count_long(g, cr, start, id, s, cnt_up, cnt_down, bad);
+  } else {
+    const unsigned e = lane < n ? mine[lane] : 0u;
+    const int j = (int)(e & 0x3ffffffu), idj = lane < n ? __ldg(id + j) : 0x7fffffff;
+    int rank = 0;
+    for (int q = 0; q < n; ++q) rank += __shfl_sync(all, idj, q) < idj;
+    const int down = __popc(__ballot_sync(all, lane < n && idj < me));
+    if (lane < n) {
+      cl.list[(long long)s * kCandKeep + rank] = e;
+      if (g.periodic) bad = shift_overflow(cr, s, j, (int)(e >> 26));
+    }
+    if (lane == 0) {
+      cnt_down[s] = down;
+      cnt_up[s] = n - down;
+    }
+  }
+  if (bad) atomicOr(err, kErrShiftRange);
+}
+
+// What the row passes read: the walk's records and lists, the bodies in slot order, the
+// new table (its ranges set) and the previous one.
+struct RowArgs {
+  CellRec cr;
+  Bodies b;
+  const Grid *grids;
+  const int *start, *new_to_old;
+  Table t, old;
+  long long N, N_old;
+  CandList cl;
+  int multi, mixed;
+};
+
+// Row r = (s, j), w the wrap of j's cell seen from s: the pair and its shift, the contact
+// history of the previous table, and in mixed precision the reference branch vector.
+__device__ inline void write_row(const RowArgs &a, int r, int s, int j, const int w[3]) {
+  const Table &nt = a.t, &ot = a.old;
+  const Grid &g = grid_of(a.grids, a.b.sid, a.multi, s);
+  int c[3] = {0, 0, 0};
+  if (g.periodic) {   // shift of body 2
+    const int4 is = a.cr.info[s], ij = a.cr.info[j];
+    c[0] = is.y - ij.y + w[0]; c[1] = is.z - ij.z + w[1]; c[2] = is.w - ij.w + w[2];
+  }
+  const int cp = pack_shift(c[0], c[1], c[2]);
+  nt.pair[r] = make_int2(s, j);
+  nt.cpack[r] = cp;
+  // both tables orient a pair by id (ids survive a collider run, or shift by the same
+  // amount within a sub-scene), so the old row is in the old range of body 1
+  int hit = -1;
+  if (ot.P > 0) {
+    const int o1 = a.new_to_old[s], o2 = a.new_to_old[j];
+    if (o1 < a.N_old && o2 < a.N_old) {
+      const int e = ot.row_start[o1 + 1];
+      for (int q = ot.row_start[o1]; q < e; ++q)
+        if (ot.pair[q].y == o2 && ot.cpack[q] == cp) { hit = q; break; }
+    }
+  }
+  const double4_32a z = make_double4_32a(0, 0, 0, 0);
+  double4_32a fs = z;
+  if (a.mixed) {
+    const float4 zf = make_float4(0, 0, 0, 0);
+    float4 hn = zf;
+    float kn = 0.0f;
+    if (hit >= 0) {
+      kn = ot.g32[hit].w;
+      if (kn != 0.0f) {
+        fs = ot.hfs[hit];
+        hn = ot.hn32[hit];
+        ot.found[hit] = 1;
+      }
+    }
+    // reference branch vector of this run, x2 + Href c - x1 formed in FP64 and rounded
+    // once to FP32; rows inside the cell have c = 0 and H c = 0 exactly, and a warp none of
+    // whose rows crosses the cell skips the conversions and products (FP64-pipe work)
+    const double4_32a p1 = a.b.pos[s], p2 = a.b.pos[j];
+    double h[3] = {0, 0, 0};
+    if (__any_sync(__activemask(), cp != 0) && g.periodic) {
+      h[0] = g.L[0] * c[0]; h[1] = g.L[1] * c[1]; h[2] = g.L[2] * c[2];
+      if (g.sheared)   // Href c of a sheared cell
+        for (int q = 0; q < 3; ++q)
+          h[q] = g.H[3 * q] * c[0] + g.H[3 * q + 1] * c[1] + g.H[3 * q + 2] * c[2];
+    }
+    const double gx = (p2.x + h[0]) - p1.x, gy = (p2.y + h[1]) - p1.y, gz = (p2.z + h[2]) - p1.z;
+    nt.g32[r] = make_float4((float)gx, (float)gy, (float)gz, kn);
+    // the squared gap of the reference configuration, in FP64 before any rounding: the
+    // mixed kernel's penetration is this minus the FP32 terms of the offsets, so it keeps
+    // FP32's relative precision of the gap rather than of the branch length
+    const double R = p1.w + p2.w;
+    nt.s0[r] = (float)(R * R - (gx * gx + gy * gy + gz * gz));
+    nt.hfs[r] = fs;
+    nt.hn32[r] = hn;
+    nt.oFM32[2 * (long long)r] = zf;
+    nt.oFM32[2 * (long long)r + 1] = zf;
+    return;
+  }
+  double4_32a hn = z;
+  double tp = 0;
+  if (hit >= 0) {
+    const double4_32a ofs = ot.hfs[hit];
+    if (ofs.w != 0.0) {
+      fs = ofs;
+      hn = ot.hn[hit];
+      tp = ot.tanphi[hit];
+      ot.found[hit] = 1;
+    }
+  }
+  nt.hfs[r] = fs;
+  nt.hn[r] = hn;
+  nt.tanphi[r] = tp;
+  nt.oFM[2 * (long long)r] = z;
+  nt.oFM[2 * (long long)r + 1] = z;
+}
+
+// The entry of a warp's 32 consecutive ranges that holds item r: lo[lane] is the first item
+// of the lane's range (ascending; all 32 lanes call).
+__device__ inline int range_of(int lo, int r) {
+  int q = 0;   // the last range that begins at or before r
+#pragma unroll
+  for (int step = 16; step > 0; step >>= 1) {
+    const int b = __shfl_sync(0xffffffffu, lo, q + step);
+    if (b <= r) q += step;
+  }
+  return q;
+}
+
+// Rows, 32 at a time: a warp takes 32 bodies, whose rows are consecutive, so every store
+// to the new table is coalesced whatever the bodies' row counts.
+__global__ void __launch_bounds__(kT) k_rows(RowArgs a) {
+  const unsigned all = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const long long base = ((long long)blockIdx.x * kT + threadIdx.x) & ~31LL;
+  if (base >= a.N) return;
+  const long long me = base + lane < a.N ? base + lane : a.N;
+  const int lo = a.t.row_start[me], hi = me < a.N ? a.t.row_start[me + 1] : lo;
+  const int nd = me < a.N ? a.t.down_start[me + 1] - a.t.down_start[me] : 0;
+  const bool listed = nd + hi - lo <= a.cl.keep;
+  const int end = __shfl_sync(all, hi, 31);
+  for (int r0 = __shfl_sync(all, lo, 0); r0 < end; r0 += 32) {
+    const int r = r0 + lane;
+    const int q = range_of(lo, r);
+    const int from = __shfl_sync(all, lo, q), skip = __shfl_sync(all, nd, q);
+    const bool mine = __shfl_sync(all, (int)listed, q);
+    if (r < end && mine) {
+      const int s = (int)base + q;
+      const unsigned e = a.cl.list[(long long)s * kCandKeep + skip + (r - from)];
+      int w[3];
+      code_wrap((int)(e >> 26), w);
+      write_row(a, r, s, (int)(e & 0x3ffffffu), w);
+    }
+  }
+  if (listed) return;
+  // more partners than a list holds: walk again, by insertion in order of id (found: the
+  // partner's id until the row is complete; cpack: its wrap)
+  const int s = (int)me, ids = a.b.id[s];
+  const Grid &g = grid_of(a.grids, a.b.sid, a.multi, s);
+  int k = lo;
+  walk_cells<false>(g, a.cr.wpos, a.start, a.cr.info[s].x, s, [&](int j, int code, float, float) {
+    const int idj = a.b.id[j];
+    if (idj < ids) return;
+    int q = k++;
+    for (; q > lo && a.t.found[q - 1] > idj; --q) {
+      a.t.found[q] = a.t.found[q - 1];
+      a.t.pair[q] = a.t.pair[q - 1];
+      a.t.cpack[q] = a.t.cpack[q - 1];
+    }
+    a.t.found[q] = idj;
+    a.t.pair[q] = make_int2(s, j);
+    a.t.cpack[q] = code;
   });
-}
-
-// Sort each body's own row range by (id of body 2, shift): the order the atomics left
-// open becomes the order of the partner ids.  Keys (the partner ids) come from the emit
-// in t.found; a range of up to kSortLocal rows is sorted in registers and local memory,
-// a longer one in place.
-constexpr int kSortLocal = 48;
-__global__ void k_rowsort(Table t, long long N) {
-  const long long sl = (long long)blockIdx.x * kT + threadIdx.x;
-  if (sl >= N) return;
-  const int r0 = t.row_start[sl], r1 = t.row_start[sl + 1], n = r1 - r0;
-  if (n < 2) return;
-  if (n <= kSortLocal) {
-    long long key[kSortLocal];   // (partner id, shift as unsigned) | position
-    int2 pr[kSortLocal];
-    int cp[kSortLocal];
-    for (int a = 0; a < n; ++a) {
-      pr[a] = t.pair[r0 + a];
-      cp[a] = t.cpack[r0 + a];
-      key[a] = ((long long)t.found[r0 + a] << 32) | (long long)(unsigned)cp[a];
-    }
-    int ord[kSortLocal];
-    for (int a = 0; a < n; ++a) {
-      int q = a - 1;
-      const long long kv = key[a];
-      while (q >= 0 && key[ord[q]] > kv) {
-        ord[q + 1] = ord[q];
-        --q;
-      }
-      ord[q + 1] = a;
-    }
-    for (int a = 0; a < n; ++a) {
-      t.pair[r0 + a] = pr[ord[a]];
-      t.cpack[r0 + a] = cp[ord[a]];
-    }
-    return;
-  }
-  for (int a = r0 + 1; a < r1; ++a) {
-    const int2 pv = t.pair[a];
-    const int cv = t.cpack[a];
-    const int kv = t.found[a];
-    int q = a - 1;
-    while (q >= r0) {
-      const int kq = t.found[q];
-      if (kq < kv || (kq == kv && (unsigned)t.cpack[q] <= (unsigned)cv)) break;
-      t.pair[q + 1] = t.pair[q];
-      t.cpack[q + 1] = t.cpack[q];
-      t.found[q + 1] = kq;
-      --q;
-    }
-    t.pair[q + 1] = pv;
-    t.cpack[q + 1] = cv;
-    t.found[q + 1] = kv;
+  for (int r = lo; r < hi; ++r) {
+    int w[3];
+    code_wrap(a.t.cpack[r], w);
+    write_row(a, r, s, a.t.pair[r].y, w);
   }
 }
 
-// After the row sort: t.found[r] = the id of body 1 of row r (the down lists' key).
-__global__ void k_rowkey(Table t, const int *__restrict__ id) {
-  const long long k = (long long)blockIdx.x * kT + threadIdx.x;
-  if (k < t.P) t.found[k] = id[t.pair[k].x];
+// the row of the pair (p, s), p the body 1
+__device__ inline int row_of(const Table &t, int p, int s) {
+  const int first = t.row_start[p], end = t.row_start[p + 1];
+  for (int r = first; r < end; ++r)
+    if (t.pair[r].y == s) return r;
+  return first;   // not reached: the walk keeps a pair from both sides or neither
 }
 
-// Down lists: every row is entered in the list of its body 2 (dfill zeroed), at a
-// position the atomics pick; k_downsort then fixes the order.
-__global__ void k_downfill(Table t, int *dfill) {
-  const long long k = (long long)blockIdx.x * kT + threadIdx.x;
-  if (k >= t.P) return;
-  const int j = t.pair[k].y;
-  const int e = t.down_start[j] + atomicAdd(&dfill[j], 1);
-  if (e < t.down_start[j + 1]) t.down[e] = (int)k;
-}
-
-// Mixed precision: the reference branch vector of every row at this run,
-// x2 + Href c - x1 formed in FP64 and rounded once to FP32.  A pass of its own over
-// the rows (one row per thread) rather than inside the emit walk, where each thread
-// meets its candidates at different iterations and the FP64 work would issue for a
-// lane or two at a time.
-__global__ void k_ref_branch(Table t, Bodies b, const Grid *__restrict__ grids, int multi) {
-  const long long k = (long long)blockIdx.x * kT + threadIdx.x;
-  if (k >= t.P) return;
-  const int2 pr = t.pair[k];
-  const Grid &g = grid_of(grids, b.sid, multi, pr.x);
-  const double4_32a p1 = b.pos[pr.x], p2 = b.pos[pr.y];
-  double h[3] = {0, 0, 0};
-  const int cp = g.periodic ? t.cpack[k] : 0;
-  // rows inside the cell have c = 0 and H c = 0 exactly: a warp none of whose rows
-  // crosses the cell skips the conversions and products (FP64-pipe instructions)
-  if (__any_sync(__activemask(), cp != 0) && g.periodic) {
-    int c0, c1, c2;
-    unpack_shift(cp, c0, c1, c2);
-    h[0] = g.L[0] * c0; h[1] = g.L[1] * c1; h[2] = g.L[2] * c2;
-    if (g.sheared)   // Href c of a sheared cell
-      for (int q = 0; q < 3; ++q) h[q] = g.H[3 * q] * c0 + g.H[3 * q + 1] * c1 + g.H[3 * q + 2] * c2;
-  }
-  const double gx = (p2.x + h[0]) - p1.x, gy = (p2.y + h[1]) - p1.y, gz = (p2.z + h[2]) - p1.z;
-  t.g32[k] = make_float4((float)gx, (float)gy, (float)gz, 0.0f);
-  // the squared gap of the reference configuration, in FP64 before any rounding: the
-  // mixed kernel's penetration is this minus the FP32 terms of the offsets, so it keeps
-  // FP32's relative precision of the gap rather than of the branch length
-  const double R = p1.w + p2.w;
-  t.s0[k] = (float)(R * R - (gx * gx + gy * gy + gz * gz));
-}
-
-// the down lists were filled in atomic order: sort each body's list by (id of body 1,
-// row); rows of one body 1 are ordered by shift within its range already.  Keys come
-// from t.found (k_rowkey); short lists are sorted in registers and local memory.
-__global__ void k_downsort(Table t, long long N) {
-  long long sl = (long long)blockIdx.x * kT + threadIdx.x;
-  if (sl >= N) return;
-  const int e0 = t.down_start[sl], e1 = t.down_start[sl + 1], n = e1 - e0;
-  if (n < 2) return;
-  if (n <= kSortLocal) {
-    long long key[kSortLocal];   // (id of body 1) << 32 | row
-    for (int a = 0; a < n; ++a) {
-      const int v = t.down[e0 + a];
-      key[a] = ((long long)t.found[v] << 32) | (long long)(unsigned)v;
+// Down lists: the rows where a body is body 2, by id of body 1, 32 entries at a time.
+__global__ void __launch_bounds__(kT) k_downs(RowArgs a) {
+  const unsigned all = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const long long base = ((long long)blockIdx.x * kT + threadIdx.x) & ~31LL;
+  if (base >= a.N) return;
+  const long long me = base + lane < a.N ? base + lane : a.N;
+  const int lo = a.t.down_start[me], hi = me < a.N ? a.t.down_start[me + 1] : lo;
+  const int nu = me < a.N ? a.t.row_start[me + 1] - a.t.row_start[me] : 0;
+  const bool listed = nu + hi - lo <= a.cl.keep;
+  const int end = __shfl_sync(all, hi, 31);
+  for (int e0 = __shfl_sync(all, lo, 0); e0 < end; e0 += 32) {
+    const int e = e0 + lane;
+    const int q = range_of(lo, e);
+    const int from = __shfl_sync(all, lo, q);
+    const bool mine = __shfl_sync(all, (int)listed, q);
+    if (e < end && mine) {
+      const int s = (int)base + q;
+      const int p = (int)(a.cl.list[(long long)s * kCandKeep + (e - from)] & 0x3ffffffu);
+      a.t.down[e] = row_of(a.t, p, s);
     }
-    for (int a = 1; a < n; ++a) {
-      const long long kv = key[a];
-      int q = a - 1;
-      while (q >= 0 && key[q] > kv) {
-        key[q + 1] = key[q];
-        --q;
-      }
-      key[q + 1] = kv;
-    }
-    for (int a = 0; a < n; ++a) t.down[e0 + a] = (int)(unsigned)(key[a] & 0xffffffffLL);
-    return;
   }
-  for (int a = e0 + 1; a < e1; ++a) {
-    const int v = t.down[a];
-    const int kv = t.found[v];
-    int b = a - 1;
-    while (b >= e0) {
-      const int u = t.down[b];
-      const int ku = t.found[u];
-      if (ku < kv || (ku == kv && u < v)) break;
-      t.down[b + 1] = u;
-      --b;
-    }
-    t.down[b + 1] = v;
-  }
+  if (listed) return;
+  const int s = (int)me, ids = a.b.id[s];
+  const Grid &g = grid_of(a.grids, a.b.sid, a.multi, s);
+  int k = lo;
+  walk_cells<false>(g, a.cr.wpos, a.start, a.cr.info[s].x, s, [&](int j, int, float, float) {
+    const int idj = a.b.id[j];
+    if (idj > ids) return;
+    int q = k++;
+    for (; q > lo && a.b.id[a.t.pair[a.t.down[q - 1]].x] > idj; --q) a.t.down[q] = a.t.down[q - 1];
+    a.t.down[q] = row_of(a.t, j, s);
+  });
 }
 
 // Integration order: bodies grouped by their number of incident rows, largest
@@ -493,63 +574,6 @@ __global__ void __launch_bounds__(kChunk) k_degree_chunk(Table t, long long N) {
   }
   __syncthreads();
   if (b >= 0) t.ord[c0 + base[b] + local] = (int)sl;
-}
-
-__global__ void k_merge(Table nt, Table ot, long long N_old, const int *__restrict__ new_to_old,
-                        int mixed) {
-  long long k = (long long)blockIdx.x * kT + threadIdx.x;
-  if (k >= nt.P) return;
-  const int2 pr = nt.pair[k];
-  const int cp = nt.cpack[k];
-  const int o1 = new_to_old[pr.x], o2 = new_to_old[pr.y];
-  // both tables orient a pair by id (ids survive a collider run, or shift by the same
-  // amount within a sub-scene), so the old row is in the old range of body 1
-  long long hit = -1;
-  if (o1 < N_old && o2 < N_old && ot.P > 0) {
-    for (int r = ot.row_start[o1]; r < ot.row_start[o1 + 1]; ++r)
-      if (ot.pair[r].y == o2 && ot.cpack[r] == cp) { hit = r; break; }
-  }
-  const double sg = 1.0;
-  if (mixed) {
-    double4_32a fs = make_double4_32a(0, 0, 0, 0);
-    float4 hn = make_float4(0, 0, 0, 0);
-    float kn = 0.0f;
-    if (hit >= 0) {
-      kn = ot.g32[hit].w;
-      if (kn != 0.0f) {
-        const double4_32a ofs = ot.hfs[hit];
-        const float4 ohn = ot.hn32[hit];
-        const float sf = (float)sg;
-        fs = make_double4_32a(sg * ofs.x, sg * ofs.y, sg * ofs.z, ofs.w);
-        hn = make_float4(sf * ohn.x, sf * ohn.y, sf * ohn.z, ohn.w);
-        ot.found[hit] = 1;
-      }
-    }
-    const float4 gref = nt.g32[k];
-    nt.g32[k] = make_float4(gref.x, gref.y, gref.z, kn);
-    nt.hfs[k] = fs;
-    nt.hn32[k] = hn;
-    nt.oFM32[2 * k] = make_float4(0, 0, 0, 0);
-    nt.oFM32[2 * k + 1] = make_float4(0, 0, 0, 0);
-    return;
-  }
-  double4_32a fs = make_double4_32a(0, 0, 0, 0), hn = make_double4_32a(0, 0, 0, 0);
-  double tp = 0;
-  if (hit >= 0) {
-    double4_32a ofs = ot.hfs[hit];
-    if (ofs.w != 0.0) {
-      double4_32a ohn = ot.hn[hit];
-      fs = make_double4_32a(sg * ofs.x, sg * ofs.y, sg * ofs.z, ofs.w);
-      hn = make_double4_32a(sg * ohn.x, sg * ohn.y, sg * ohn.z, ohn.w);
-      tp = ot.tanphi[hit];
-      ot.found[hit] = 1;
-    }
-  }
-  nt.hfs[k] = fs;
-  nt.hn[k] = hn;
-  nt.tanphi[k] = tp;
-  nt.oFM[2 * k] = make_double4_32a(0, 0, 0, 0);
-  nt.oFM[2 * k + 1] = make_double4_32a(0, 0, 0, 0);
 }
 
 // A real row of the previous table that no candidate carried over: an error only
@@ -598,73 +622,49 @@ void launch_bbox_sub(const Bodies &b, long long N, int cap, unsigned long long *
 }
 
 void launch_bin(const Bodies &b, long long N, const Grid *grids, int multi, uint32_t dead,
-                uint32_t *key, int *count, cudaStream_t st) {
-  if (N > 0) k_bin<<<blocks(N), kT, 0, st>>>(b.pos, b.sid, N, grids, multi, dead, key, count);
+                uint32_t *key, int *rank, int *count, CellRec raw, cudaStream_t st) {
+  if (N > 0)
+    k_bin<<<blocks(N), kT, 0, st>>>(b.pos, b.sid, N, grids, multi, dead, key, rank, count, raw);
 }
 
-void launch_scatter(long long N, const uint32_t *key, const int *start, int *fill, int *tmp,
+void launch_scatter(long long N, const uint32_t *key, const int *rank, const int *start, int *tmp,
                     cudaStream_t st) {
-  if (N > 0) k_scatter<<<blocks(N), kT, 0, st>>>(N, key, start, fill, tmp);
-}
-
-void launch_cellsort(const int *count, const int *start, long long ncell, const int *id,
-                     int *tmp, cudaStream_t st) {
-  k_cellsort<<<blocks(ncell), kT, 0, st>>>(count, start, ncell, id, tmp);
+  if (N > 0) k_scatter<<<blocks(N), kT, 0, st>>>(N, key, rank, start, tmp);
 }
 
 void launch_reorder(const Bodies &src, const Bodies &dst, long long N, long long cap,
-                    const int *new_to_old, int *slot_of_id, int has_walls, int mixed,
-                    const int *id_shift, cudaStream_t st) {
+                    const int *tmp, const uint32_t *key, const int *start, CellRec raw, CellRec cr,
+                    int *new_to_old, int *slot_of_id, int has_walls,
+                    int mixed, const int *id_shift, cudaStream_t st) {
   if (N > 0)
-    k_reorder<<<blocks(N), kT, 0, st>>>(src, dst, N, cap, new_to_old, slot_of_id, has_walls,
-                                        mixed, id_shift);
+    k_reorder<<<blocks(N), kT, 0, st>>>(src, dst, N, cap, tmp, key, start, raw, cr,
+                                        new_to_old, slot_of_id, has_walls, mixed, id_shift);
 }
 
-void launch_cellrec(const Bodies &b, long long N, const Grid *grids, int multi, float4 *wpos,
-                    int4 *info, cudaStream_t st) {
-  if (N > 0) k_cellrec<<<blocks(N), kT, 0, st>>>(b.pos, b.sid, N, grids, multi, CellRec{wpos, info});
-}
-
-void launch_count(float4 *wpos, int4 *info, const int *sid, const int *id, long long N,
-                  const Grid *grids, int multi, const int *count, const int *start, int *cnt_up,
-                  int *cnt_down, int *err, CandList cl, cudaStream_t st) {
-  if (N > 0)
-    k_count<<<blocks(N), kT, 0, st>>>(CellRec{wpos, info}, sid, id, N, grids, multi, count, start,
-                                      cnt_up, cnt_down, err, cl);
-}
-
-void launch_emit(float4 *wpos, int4 *info, const Bodies &b, long long N, const Grid *grids,
-                 int multi, const int *count, const int *start, const Table &t, int *ufill,
-                 int *dfill, CandList cl, cudaStream_t st) {
+void launch_partners(CellRec cr, const int *sid, const int *id, long long N, const Grid *grids,
+                     int multi, const int *start, int *cnt_up, int *cnt_down, int *err, CandList cl,
+                     cudaStream_t st) {
   if (N <= 0) return;
-  k_emit<<<blocks(N), kT, 0, st>>>(CellRec{wpos, info}, b, N, grids, multi, count, start, t,
-                                   ufill, cl);
-  k_rowsort<<<blocks(N), kT, 0, st>>>(t, N);
-  if (t.P > 0) {
-    k_rowkey<<<blocks(t.P), kT, 0, st>>>(t, b.id);
-    k_downfill<<<blocks(t.P), kT, 0, st>>>(t, dfill);
-  }
+  if (N < kWarpBodies)
+    k_partners_warp<<<blocks(32 * N), kT, 0, st>>>(cr, sid, id, N, grids, multi, start, cnt_up,
+                                                   cnt_down, err, cl);
+  else
+    k_partners<<<(unsigned)((N + kPT - 1) / kPT), kPT, 0, st>>>(cr, sid, id, N, grids, multi, start,
+                                                               cnt_up, cnt_down, err, cl);
 }
 
-void launch_ref_branch(const Table &t, const Bodies &b, const Grid *grids, int multi,
-                       cudaStream_t st) {
-  if (t.P > 0) k_ref_branch<<<blocks(t.P), kT, 0, st>>>(t, b, grids, multi);
-}
-
-void launch_downsort(const Table &t, const int *id, long long N, cudaStream_t st) {
-  (void)id;   // the keys are in t.found (k_rowkey)
-  if (N > 0) k_downsort<<<blocks(N), kT, 0, st>>>(t, N);
-}
-
-void launch_degree_order(const Table &t, long long N, int *ws, cudaStream_t st) {
+void launch_rows(CellRec cr, const Bodies &b, const Grid *grids, int multi, const int *start,
+                 const Table &nt, const Table &ot, long long N, long long N_old,
+                 const int *new_to_old, CandList cl, int mixed, cudaStream_t st) {
   if (N <= 0) return;
-  (void)ws;
+  const RowArgs a{cr, b, grids, start, new_to_old, nt, ot, N, N_old, cl, multi, mixed};
+  k_rows<<<blocks(N), kT, 0, st>>>(a);
+  k_downs<<<blocks(N), kT, 0, st>>>(a);
+}
+
+void launch_degree_order(const Table &t, long long N, cudaStream_t st) {
+  if (N <= 0) return;
   k_degree_chunk<<<(unsigned)((N + kChunk - 1) / kChunk), kChunk, 0, st>>>(t, N);
-}
-
-void launch_merge(const Table &nt, const Table &ot, long long N_old, const int *new_to_old,
-                  int mixed, cudaStream_t st) {
-  if (nt.P > 0) k_merge<<<blocks(nt.P), kT, 0, st>>>(nt, ot, N_old, new_to_old, mixed);
 }
 
 namespace {

@@ -256,53 +256,49 @@ void exclusive_scan2(const int *in0, int *out0, const int *in1, int *out1, long 
 // collider.cu
 void launch_bbox(const Bodies &b, long long N, double *partials, int nblk, cudaStream_t st);
 int bbox_blocks(long long N);
+// Per-body collider record: FP32 position relative to the grid (periodic: the wrapped
+// position), radius, packed cell coordinates and the integer image.
+struct CellRec {
+  float4 *wpos;   // (x, y, z, r)
+  int4 *info;     // (cell0 | cell1 << 10 | cell2 << 20, img0, img1, img2)
+};
 // grids: device array, one per sub-scene (multi) or one; bodies whose grid has no
-// cells take the key `dead`
+// cells take the key `dead`.  rank: the body's place among its cell's arrivals; raw: its
+// record, in the order of the bodies before the run
 void launch_bin(const Bodies &b, long long N, const Grid *grids, int multi, uint32_t dead,
-                uint32_t *key, int *count, cudaStream_t st);
-void launch_scatter(long long N, const uint32_t *key, const int *start, int *fill, int *tmp,
+                uint32_t *key, int *rank, int *count, CellRec raw, cudaStream_t st);
+// tmp: bodies cell by cell, in order of arrival within a cell
+void launch_scatter(long long N, const uint32_t *key, const int *rank, const int *start, int *tmp,
                     cudaStream_t st);
-void launch_cellsort(const int *count, const int *start, long long ncell, const int *id,
-                     int *tmp, cudaStream_t st);
+// bodies and records to their slots (by id within a cell)
 // id_shift (nullable): per sub-scene amount subtracted from the ids (removals)
 void launch_reorder(const Bodies &src, const Bodies &dst, long long N, long long cap,
-                    const int *new_to_old, int *slot_of_id, int has_walls, int mixed,
+                    const int *tmp, const uint32_t *key, const int *start, CellRec raw, CellRec cr,
+                    int *new_to_old, int *slot_of_id, int has_walls, int mixed,
                     const int *id_shift, cudaStream_t st);
 // per-sub-scene bounding boxes as ordered keys (see collider.cu); keys preset
 void launch_bbox_sub(const Bodies &b, long long N, int cap, unsigned long long *keys, int nsm,
                      cudaStream_t st);
-void launch_cellrec(const Bodies &b, long long N, const Grid *grids, int multi, float4 *wpos,
-                    int4 *info, cudaStream_t st);
-// cnt_up / cnt_down: zeroed; counts of the rows of each body as body 1 / body 2 (body 1:
-// the smaller id)
-// The count pass keeps up to kCandKeep candidates per walker (partner slot and the
-// wrap of its neighbour cell, packed in 32 bits) in a scratch list, and their number;
-// the emit pass places those without walking the cells again (a walker with more, or
-// slots beyond 2^26, walks again).
+// Partners of a body, up to kCandKeep (slot and the wrap of the partner's cell, packed in
+// 32 bits), by id: those of smaller id, then those of larger id.  keep: kCandKeep, or 0
+// where slots do not fit 26 bits; a body with more partners has no list and is walked
+// again by the row passes.
 constexpr int kCandKeep = 32;
 struct CandList {
-  unsigned *list;   // kCandKeep entries per body: slot | wrap code << 26
-  int *n;           // candidates the walker found (may exceed kCandKeep)
-  int use;          // 0: slots too large to pack, emit walks
+  unsigned *list;
+  int keep;
 };
-void launch_count(float4 *wpos, int4 *info, const int *sid, const int *id, long long N,
-                  const Grid *grids, int multi, const int *count, const int *start, int *cnt_up,
-                  int *cnt_down, int *err, CandList cl, cudaStream_t st);
-// rows in body 1's range sorted by body 2's id, and the down lists filled (unsorted);
-// ufill, dfill: zeroed; cl: the count pass's candidates
-void launch_emit(float4 *wpos, int4 *info, const Bodies &b, long long N, const Grid *grids,
-                 int multi, const int *count, const int *start, const Table &t, int *ufill,
-                 int *dfill, CandList cl, cudaStream_t st);
-// each down list sorted by body 1's id
-void launch_downsort(const Table &t, const int *id, long long N, cudaStream_t st);
-// t.ord = bodies in decreasing order of incident rows; ws: 2 * kDegreeBuckets zeroed ints
-void launch_degree_order(const Table &t, long long N, int *ws, cudaStream_t st);
-void launch_merge(const Table &nt, const Table &ot, long long N_old, const int *new_to_old,
-                  int mixed, cudaStream_t st);
-// mixed tables: reference branch vectors (g32.xyz) and squared reference gaps (s0) of
-// every row, after the emit
-void launch_ref_branch(const Table &t, const Bodies &b, const Grid *grids, int multi,
-                       cudaStream_t st);
+// cnt_up / cnt_down: partners of larger / smaller id of every body
+void launch_partners(CellRec cr, const int *sid, const int *id, long long N, const Grid *grids,
+                     int multi, const int *start, int *cnt_up, int *cnt_down, int *err, CandList cl,
+                     cudaStream_t st);
+// rows (with the history of the old table: `found` marks the rows carried over) and down
+// lists of the new table, whose row_start and down_start are set
+void launch_rows(CellRec cr, const Bodies &b, const Grid *grids, int multi, const int *start,
+                 const Table &nt, const Table &ot, long long N, long long N_old,
+                 const int *new_to_old, CandList cl, int mixed, cudaStream_t st);
+// t.ord = bodies in decreasing order of incident rows within runs of slots
+void launch_degree_order(const Table &t, long long N, cudaStream_t st);
 void launch_lost(const Table &ot, const Bodies &ob, const Grid *grids, int multi, int *err,
                  int mixed, cudaStream_t st);
 // cell flip: rows of sub-scene `sub` (all rows unless multi) get c' = Minv c (apply = 1),

@@ -1,7 +1,6 @@
 // Uniform-grid helpers shared by the collider (collider.cu) and the bare pair
 // query (pairs.cu): Morton codes of cells, the cell and integer image of a
-// position, the forward half of the 27-cell stencil, and the conservative FP32
-// candidate test.
+// position, the conservative FP32 candidate test and the walk of the 27-cell stencil.
 #pragma once
 #include "dem_internal.cuh"
 
@@ -56,106 +55,43 @@ __device__ inline int neg_shift(int p) {
   return pack_shift(-a, -b, -c);
 }
 
-// Forward half of the 27-cell stencil: own cell (partners with a higher slot)
-// plus the 13 offsets with (dz, dy, dx) lexicographically positive, so every pair
-// of neighbouring cells is visited from exactly one side.
-template <class F>
-__device__ inline void for_half_shell(const Grid &g, const int *__restrict__ count,
-                                      const int *__restrict__ start, const int ci[3], int s,
-                                      F &&f) {
-  for (int dz = 0; dz <= 1; ++dz)
-    for (int dy = (dz ? -1 : 0); dy <= 1; ++dy)
-      for (int dx = ((dz || dy) ? -1 : 0); dx <= 1; ++dx) {
-        const int d[3] = {dx, dy, dz};
-        int cj[3], w[3];
-        bool ok = true;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          int c = ci[k] + d[k];
-          w[k] = 0;
-          if (g.periodic) {
-            if (c < 0) { c += g.n[k]; w[k] = -1; }
-            else if (c >= g.n[k]) { c -= g.n[k]; w[k] = 1; }
-          } else if (c < 0 || c >= g.n[k]) {
-            ok = false;
-          }
-          cj[k] = c;
-        }
-        if (!ok) continue;
-        const bool self = (dx == 0 && dy == 0 && dz == 0);
-        const long long m = cell_index(g, cj[0], cj[1], cj[2]);
-        const int s0 = start[m], cnt = count[m];
-        for (int j = (self ? s + 1 : s0); j < s0 + cnt; ++j) f(j, w);
-      }
-}
-
-// Per-slot collider record: FP32 position relative to the grid (periodic: the
-// wrapped position), radius, packed cell coordinates and the integer image.
-struct CellRec {
-  float4 *wpos;   // (x, y, z, r)
-  int4 *info;     // (cell0 | cell1 << 10 | cell2 << 20, img0, img1, img2)
-};
-
-// Conservative FP32 candidate test of (s, j): keeps every pair whose FP64
-// distance is below r1 + r2 + reach (the slack covers the FP32 rounding of
-// coordinates bounded by the cell size), so the candidate set is a superset of
-// the exact one; count and emit evaluate it identically.
-__device__ inline bool cand_f32(const Grid &g, const float4 &a, const float4 &b, const int w[3],
-                                float slack) {
-  float sx = (float)w[0] * g.Lf[0], sy = (float)w[1] * g.Lf[1], sz = (float)w[2] * g.Lf[2];
-  if (g.sheared) {   // image shift H w of a sheared cell
-    const float f0 = (float)w[0], f1 = (float)w[1], f2 = (float)w[2];
-    sx = g.Hf[0] * f0 + g.Hf[1] * f1 + g.Hf[2] * f2;
-    sy = g.Hf[3] * f0 + g.Hf[4] * f1 + g.Hf[5] * f2;
-    sz = g.Hf[6] * f0 + g.Hf[7] * f1 + g.Hf[8] * f2;
-  }
-  const float dx = (b.x + sx) - a.x;
-  const float dy = (b.y + sy) - a.y;
-  const float dz = (b.z + sz) - a.z;
-  const float R = (a.w + b.w) + g.reachf + slack;
-  return dx * dx + dy * dy + dz * dz < R * R;
-}
-
-// ---- one warp per cell
-//
-// A thread per body walks the neighbour cells with every lane of its warp in another
-// cell: the lanes wait for the one with the fullest cells, each cell costs every lane
-// its own address arithmetic and two dependent loads, and what a lane does with a hit is
-// issued for a lane or two at a time.  Here a warp takes a cell: its lanes fetch the
-// ranges of the neighbour cells together (one round of loads), the partners of all of
-// them are laid end to end and loaded 32 at a time, and each chunk is tested against
-// every body of the cell.  A chunk's hits keep the stencil order (dz, dy, dx, slot), so
-// their positions in a body's list come from a ballot and the lists are the ones the
-// per-thread walk gives.
-
-constexpr int kStencil = 27;
-
-// Neighbour cell t (0..26, dx fastest) of cell ci: its bodies and its wrap (code 0..26);
-// no bodies beyond the faces of an aperiodic grid.
-__device__ inline void stencil_cell(const Grid &g, const int *__restrict__ count,
-                                    const int *__restrict__ start, const int ci[3], int t,
-                                    int &first, int &cnt, int &code) {
-  const int d[3] = {t % 3 - 1, (t / 3) % 3 - 1, t / 9 - 1};
-  int cj[3], w[3];
-  bool ok = true;
+// Image shift of the cells of wrap w, in FP32 (H w of a sheared cell): the shift of -w is
+// its exact negative.
+__device__ inline void wrap_shift_f32(const Grid &g, const int w[3], float sh[3]) {
+  const float f0 = (float)w[0], f1 = (float)w[1], f2 = (float)w[2];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    int c = ci[k] + d[k];
-    w[k] = 0;
-    if (g.periodic) {
-      if (c < 0) { c += g.n[k]; w[k] = -1; }
-      else if (c >= g.n[k]) { c -= g.n[k]; w[k] = 1; }
-    } else if (c < 0 || c >= g.n[k]) {
-      ok = false;
-      c = 0;
-    }
-    cj[k] = c;
+    if (g.sheared)
+      sh[k] = __fmaf_rn(g.Hf[3 * k + 2], f2, __fmaf_rn(g.Hf[3 * k + 1], f1, __fmul_rn(g.Hf[3 * k], f0)));
+    else
+      sh[k] = __fmul_rn(k == 0 ? f0 : (k == 1 ? f1 : f2), g.Lf[k]);
   }
-  const long long m = cell_index(g, cj[0], cj[1], cj[2]);
-  first = ok ? start[m] : 0;
-  cnt = ok ? count[m] : 0;
-  code = (w[0] + 1) + 3 * (w[1] + 1) + 9 * (w[2] + 1);
 }
+
+// Conservative FP32 candidate test of (s, j): keeps every pair whose FP64 distance is
+// below r1 + r2 + reach (the slack covers the FP32 rounding of coordinates bounded by the
+// cell size), so the candidate set is a superset of the exact one.  A pair met from both
+// sides must be decided alike, so the image shift goes to the same of the two spheres
+// from either side (to the partner of wrap code above 13; code and 26 - code are opposite
+// wraps) and every operation is written out: no contraction that differs by call site.
+__device__ inline float3 placed_f32(const float4 &b, const float sh[3], int code) {
+  return code > 13 ? make_float3(__fadd_rn(b.x, sh[0]), __fadd_rn(b.y, sh[1]), __fadd_rn(b.z, sh[2]))
+                   : make_float3(b.x, b.y, b.z);
+}
+__device__ inline float3 moved_f32(const float sh[3], int code) {   // what the body itself moves by
+  return code < 13 ? make_float3(-sh[0], -sh[1], -sh[2]) : make_float3(0.0f, 0.0f, 0.0f);
+}
+__device__ inline bool cand_f32(const float3 &a, float ra, const float3 &b, float rb, float reach,
+                                float &d2, float &R) {   // a, b placed; reach = cand_reach(g)
+  const float dx = __fsub_rn(b.x, a.x), dy = __fsub_rn(b.y, a.y), dz = __fsub_rn(b.z, a.z);
+  R = __fadd_rn(__fadd_rn(ra, rb), reach);
+  d2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
+  return d2 < __fmul_rn(R, R);
+}
+__device__ inline float cand_reach(const Grid &g) { return __fadd_rn(g.reachf, g.slack); }
+
+constexpr int kStencil = 27;
+constexpr int kNoWrap = 13;   // wrap code of no wrap at all: (w0 + 1) + 3 (w1 + 1) + 9 (w2 + 1)
 
 __device__ inline void code_wrap(int code, int w[3]) {
   w[0] = code % 3 - 1;
@@ -163,87 +99,112 @@ __device__ inline void code_wrap(int code, int w[3]) {
   w[2] = code / 9 - 1;
 }
 
-// Image shift of the cells of wrap w in FP32, as cand_f32 forms it.
-__device__ inline void wrap_shift_f32(const Grid &g, const int w[3], float &sx, float &sy,
-                                      float &sz) {
-  const float f0 = (float)w[0], f1 = (float)w[1], f2 = (float)w[2];
-  sx = f0 * g.Lf[0]; sy = f1 * g.Lf[1]; sz = f2 * g.Lf[2];
-  if (g.sheared) {
-    sx = g.Hf[0] * f0 + g.Hf[1] * f1 + g.Hf[2] * f2;
-    sy = g.Hf[3] * f0 + g.Hf[4] * f1 + g.Hf[5] * f2;
-    sz = g.Hf[6] * f0 + g.Hf[7] * f1 + g.Hf[8] * f2;
-  }
+// One axis of a stencil cell: coordinate c (outside the grid by at most one) wrapped or
+// refused, and its part of the cell index.
+__device__ inline bool axis_cell(const Grid &g, int k, int &c, int &w) {
+  w = 0;
+  if (c >= 0 && c < g.n[k]) return true;
+  if (!g.periodic) return false;
+  w = c < 0 ? -1 : 1;
+  c -= w * g.n[k];
+  return true;
+}
+__device__ inline int axis_part(const Grid &g, int k, int c) {
+  if (g.morton) return (int)(spread3((uint32_t)c) << k);
+  return k == 0 ? c : (k == 1 ? c * g.n[0] : c * g.n[0] * g.n[1]);
 }
 
-// The walk of one cell by one warp: cnt bodies from slot s0, cell coordinates ci.
-//   kFull: all 27 cells (each pair met from both sides), else the forward half shell
-//   test(s, j, code, d2, R): the pair's decision from its FP32 squared distance and reach
-//   hit(s, j, code, pos): called by the lane of a kept pair, pos its place in s's list
-//   done(s, n): called by lane h of a group of up to 32 bodies, n the kept pairs of body s
-//               (after a __syncwarp: what the hits wrote is visible to the warp)
-template <bool kFull, class Test, class Hit, class Done>
-__device__ inline void warp_walk(const Grid &g, const float4 *__restrict__ wpos,
-                                 const int *__restrict__ count, const int *__restrict__ start,
-                                 int s0, int cnt, const int ci[3], Test &&test, Hit &&hit,
-                                 Done &&done) {
-  const unsigned all = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  const int nst = kFull ? kStencil : kStencil / 2 + 1;
-  int first = 0, num = 0, code = 0;
-  if (lane < nst)
-    stencil_cell(g, count, start, ci, kFull ? lane : kStencil / 2 + lane, first, num, code);
-  int incl = num;
+// Neighbour cell t (0..26, dx fastest) of cell ci: its slots [first, end) and wrap code;
+// none beyond the faces of an aperiodic grid.
+__device__ inline void stencil_cell(const Grid &g, const int *__restrict__ start, const int ci[3],
+                                    int t, int &first, int &end, int &code) {
+  int c[3] = {ci[0] + t % 3 - 1, ci[1] + (t / 3) % 3 - 1, ci[2] + t / 9 - 1}, w[3];
+  bool ok = true;
+  for (int k = 0; k < 3; ++k) ok = axis_cell(g, k, c[k], w[k]) && ok;
+  const long long m =
+      ok ? g.base + axis_part(g, 0, c[0]) + axis_part(g, 1, c[1]) + axis_part(g, 2, c[2]) : 0;
+  first = ok ? start[m] : 0;
+  end = ok ? start[m + 1] : 0;
+  code = (w[0] + 1) + 3 * (w[1] + 1) + 9 * (w[2] + 1);
+}
+
+// Walk of one body's neighbour cells by one thread, in stencil order (dz, dy, dx, slot):
+// f(j, code, d2, R) for every candidate j (FP32 squared distance, reach with slack).
+//   kHalf: the forward half of the stencil (own cell from slot s + 1 on, then the 13 cells
+//   with (dz, dy, dx) lexicographically positive), so every pair is met from one side;
+//   else all 27 cells, the body itself left out: every pair is met from both sides.
+// A cell costs its index and two loads (the three of a row together), a partner about 17
+// instructions and a load; kAhead partners are loaded before the first is tested.  Loading
+// one at a time left the walk waiting: all 27 cells of 300k bodies at three rows a body
+// 136 -> 111 us, of 1M bodies at five 852 -> 605 us with four ahead (118 and 697 with
+// two); the half shell of 1M bodies 236 -> 219 us with two (254 with four).  Where cells run
+// along x in memory (row-major grids), the three cells of a row inside the grid are one run.
+template <bool kHalf, class F>
+__device__ inline void walk_cells(const Grid &g, const float4 *__restrict__ wpos,
+                                  const int *__restrict__ start, int packed, int s, F &&f) {
+  constexpr int kAhead = kHalf ? 2 : 4;
+  const float4 me = wpos[s];
+  const float reach = cand_reach(g);
+  const int ci[3] = {packed & 1023, (packed >> 10) & 1023, (packed >> 20) & 1023};
+  bool okx[3];
+  int px[3], wx[3];
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(all, incl, o);
-    if (lane >= o) incl += y;
+  for (int i = 0; i < 3; ++i) {
+    int c = ci[0] + i - 1;
+    okx[i] = axis_cell(g, 0, c, wx[i]);
+    px[i] = okx[i] ? axis_part(g, 0, c) : 0;
   }
-  const int total = __shfl_sync(all, incl, 31);
-  for (int h0 = 0; h0 < cnt; h0 += 32) {
-    const int hb = min(32, cnt - h0);
-    int mine = 0;   // lane h: kept pairs of body s0 + h0 + h so far
-    for (int c0 = 0; c0 < total; c0 += 32) {
-      const int t = c0 + lane;
-      int q = 0;   // the cell of partner t: the number of cells that end at or before t
+  const bool run = !kHalf && !g.morton && wx[0] == 0 && wx[2] == 0;
+#pragma unroll 1
+  for (int dz = kHalf ? 0 : -1; dz <= 1; ++dz) {
+    int cz = ci[2] + dz, wz;
+    if (!axis_cell(g, 2, cz, wz)) continue;
+    const long long pz = g.base + axis_part(g, 2, cz);
+#pragma unroll 1
+    for (int dy = kHalf && dz == 0 ? 0 : -1; dy <= 1; ++dy) {
+      int cy = ci[1] + dy, wy;
+      if (!axis_cell(g, 1, cy, wy)) continue;
+      const long long row = pz + axis_part(g, 1, cy);
+      const bool own_row = dz == 0 && dy == 0;
+      int a[3], b[3];
 #pragma unroll
-      for (int step = 16; step > 0; step >>= 1) {
-        const int e = __shfl_sync(all, incl, q + step - 1);
-        if (e <= t) q += step;
-      }
-      q = min(q, 31);
-      const int j = __shfl_sync(all, first, q) + t - (__shfl_sync(all, incl, q) - __shfl_sync(all, num, q));
-      const int cj = __shfl_sync(all, code, q);
-      const bool valid = t < total;
-      const bool own = q == (kFull ? kStencil / 2 : 0);
-      float4 b = make_float4(0, 0, 0, 0);
-      if (valid) {
-        b = __ldg(wpos + j);
-        if (g.periodic && cj != kStencil / 2) {
-          int w[3];
-          float sx, sy, sz;
-          code_wrap(cj, w);
-          wrap_shift_f32(g, w, sx, sy, sz);
-          b.x += sx; b.y += sy; b.z += sz;
+      for (int i = 0; i < 3; ++i) {
+        a[i] = b[i] = 0;
+        if (okx[i] && !(kHalf && own_row && i == 0)) {
+          a[i] = start[row + px[i]];
+          b[i] = start[row + px[i] + 1];
         }
       }
-      for (int h = 0; h < hb; ++h) {
-        const int s = s0 + h0 + h;
-        const float4 a = __ldg(wpos + s);
-        const float dx = b.x - a.x, dy = b.y - a.y, dz = b.z - a.z;
-        const float R = (a.w + b.w) + g.reachf + g.slack;
-        const float d2 = dx * dx + dy * dy + dz * dz;
-        bool keep = valid && d2 < R * R && !(own && (kFull ? j == s : j <= s));
-        if (keep) keep = test(s, j, cj, d2, R);
-        const unsigned m = __ballot_sync(all, keep);
-        if (m) {
-          const int at = __shfl_sync(all, mine, h);
-          if (keep) hit(s, j, cj, at + __popc(m & ((1u << lane) - 1u)));
-          if (lane == h) mine += __popc(m);
+      if (kHalf && own_row) a[1] = s + 1;
+      if (run) {   // one run of slots
+        if (okx[0]) a[1] = a[0];
+        if (okx[2]) b[1] = b[2];
+        a[0] = b[0] = a[2] = b[2] = 0;
+      }
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const int code = (wx[i] + 1) + 3 * (wy + 1) + 9 * (wz + 1);
+        float3 at = make_float3(me.x, me.y, me.z);
+        float sh[3] = {0, 0, 0};
+        if (code != kNoWrap) {
+          const int w[3] = {wx[i], wy, wz};
+          wrap_shift_f32(g, w, sh);
+          const float3 mv = moved_f32(sh, code);
+          at = make_float3(__fadd_rn(me.x, mv.x), __fadd_rn(me.y, mv.y), __fadd_rn(me.z, mv.z));
+        }
+        for (int j = a[i]; j < b[i]; j += kAhead) {
+          float4 p[kAhead];
+#pragma unroll
+          for (int q = 0; q < kAhead; ++q) p[q] = __ldg(wpos + min(j + q, b[i] - 1));
+#pragma unroll
+          for (int q = 0; q < kAhead; ++q) {
+            float d2, R;
+            const bool near = cand_f32(at, me.w, placed_f32(p[q], sh, code), p[q].w, reach, d2, R);
+            if (near && j + q < b[i] && (kHalf || j + q != s)) f(j + q, code, d2, R);
+          }
         }
       }
     }
-    __syncwarp();
-    done(s0 + h0 + lane, mine, lane < hb);
   }
 }
 

@@ -4,8 +4,8 @@
 // then the exact sphere test) without a scene.
 //
 // Same grid as the scene collider: spheres are binned by Morton cell and sorted by a
-// counting sort (by index within a cell); a warp takes a cell and scans the forward half
-// of its 27-cell neighbourhood (grid.cuh).  The FP32 distance decides every pair that is
+// counting sort (by index within a cell); each one scans the forward half of its 27-cell
+// neighbourhood (grid.cuh).  The FP32 distance decides every pair that is
 // not within its rounding allowance of the threshold; the others pass the exact FP64
 // test |x_j + H c - x_i| < (r_i + r_j) + margin, evaluated with round-to-nearest
 // operations in the order written (shift, branch vector, squared length left to right),
@@ -116,15 +116,14 @@ __global__ void k_scatter_q(long long n, const uint32_t *__restrict__ key,
 // that order open).  The records of a cell's members are read by its neighbours in the
 // warp as well, so the count of smaller indices costs no memory traffic to speak of.
 __global__ void k_place(long long n, const int *__restrict__ tmp, const uint32_t *__restrict__ key,
-                        const int *__restrict__ count, const int *__restrict__ start, CellRec raw,
-                        int *order, CellRec cr) {
+                        const int *__restrict__ start, CellRec raw, int *order, CellRec cr) {
   long long p = (long long)blockIdx.x * kT + threadIdx.x;
   if (p >= n) return;
   const int i = tmp[p];
   const uint32_t m = key[i];
-  const int st = start[m], cnt = count[m];
-  int s = st;
-  for (int q = 0; q < cnt; ++q) s += tmp[st + q] < i;
+  const int first = start[m], end = start[m + 1];
+  int s = first;
+  for (int q = first; q < end; ++q) s += tmp[q] < i;
   order[s] = i;
   cr.wpos[s] = raw.wpos[i];
   cr.info[s] = raw.info[i];
@@ -152,7 +151,7 @@ struct PairView {
   const double *pos, *rad;   // the caller's
   const int *order;          // index of the sphere in each slot
   CellRec cr;
-  const int *count, *start;
+  const int *start;
   double margin;
   long long n;
 };
@@ -192,38 +191,23 @@ __device__ inline bool is_pair(const PairView &v, const Grid &g, int s, int j, c
 constexpr int kPairKeep = 16;
 constexpr long long kPairSlots = 1LL << 26;
 
-// Count pass, a warp per cell (`per` consecutive cells to a warp, so that large grids,
-// where most cells hold a sphere or none, need no warp for each).  The walk is bound by
-// instruction issue and the latency of the cell ranges.  A million spheres at solid
-// fraction 0.62, whole query: 4.15 -> 0.62 ms; 3001 spheres: 0.35 -> 0.17 ms.
-__global__ void __launch_bounds__(kT) k_pair_count(PairView v, Grid g, long long ncell, int per,
-                                                   unsigned *list, int keep, int *cnt) {
-  const int lane = threadIdx.x & 31;
-  const long long base = (((long long)blockIdx.x * kT + threadIdx.x) >> 5) * per;
-  int num = 0, first = 0;
-  if (lane < per && base + lane < ncell) {
-    num = v.count[base + lane];
-    first = v.start[base + lane];
-  }
-  unsigned todo = __ballot_sync(0xffffffffu, num > 0);
-  while (todo) {
-    const int b = __ffs(todo) - 1;
-    todo &= todo - 1;
-    const int s0 = __shfl_sync(0xffffffffu, first, b), k = __shfl_sync(0xffffffffu, num, b);
-    const int packed = v.cr.info[s0].x;
-    const int ci[3] = {packed & 1023, (packed >> 10) & 1023, (packed >> 20) & 1023};
-    warp_walk<false>(
-        g, v.cr.wpos, v.count, v.start, s0, k, ci,
-        [&](int s, int j, int code, float d2, float R) {
-          int w[3];
-          code_wrap(code, w);
-          return is_pair(v, g, s, j, w, d2, R);
-        },
-        [&](int s, int j, int code, int at) {
-          if (at < keep) list[(long long)s * kPairKeep + at] = (unsigned)j | ((unsigned)code << 26);
-        },
-        [&](int s, int n, bool own) { if (own) cnt[s] = n; });
-  }
+// Count pass, a thread per slot.  A million spheres at solid fraction 0.62, whole query:
+// 4.15 -> 0.58 ms; 3001 spheres: 0.35 -> 0.17 ms.
+__global__ void __launch_bounds__(kT) k_pair_count(PairView v, Grid g, unsigned *list, int keep,
+                                                   int *cnt) {
+  const long long sl = (long long)blockIdx.x * kT + threadIdx.x;
+  if (sl >= v.n) return;
+  const int s = (int)sl;
+  int n = 0;
+  unsigned *mine = list + sl * kPairKeep;
+  walk_cells<true>(g, v.cr.wpos, v.start, v.cr.info[s].x, s, [&](int j, int code, float d2, float R) {
+    int w[3];
+    code_wrap(code, w);
+    if (!is_pair(v, g, s, j, w, d2, R)) return;
+    if (n < keep) mine[n] = (unsigned)j | ((unsigned)code << 26);
+    ++n;
+  });
+  cnt[s] = n;
 }
 
 struct PairOut {
@@ -276,18 +260,11 @@ __global__ void __launch_bounds__(kT) k_pair_emit(PairView v, Grid g, const unsi
   }
   if (!listed) {
     const int s = (int)me;
-    const float4 a = v.cr.wpos[s];
-    const int packed = v.cr.info[s].x;
-    const int ci[3] = {packed & 1023, (packed >> 10) & 1023, (packed >> 20) & 1023};
     long long r = lo;
-    for_half_shell(g, v.count, v.start, ci, s, [&](int j, const int w[3]) {
-      const float4 b = v.cr.wpos[j];
-      float sx, sy, sz;
-      wrap_shift_f32(g, w, sx, sy, sz);
-      const float dx = (b.x + sx) - a.x, dy = (b.y + sy) - a.y, dz = (b.z + sz) - a.z;
-      const float R = (a.w + b.w) + g.reachf + g.slack;
-      const float d2 = dx * dx + dy * dy + dz * dz;
-      if (d2 < R * R && is_pair(v, g, s, j, w, d2, R)) put_pair(v, g, o, r++, s, j, w);
+    walk_cells<true>(g, v.cr.wpos, v.start, v.cr.info[s].x, s, [&](int j, int code, float d2, float R) {
+      int w[3];
+      code_wrap(code, w);
+      if (is_pair(v, g, s, j, w, d2, R)) put_pair(v, g, o, r++, s, j, w);
     });
   }
 }
@@ -416,20 +393,16 @@ void pairs_extent(const double *pos, const double *rad, long long n, const PairS
 // Second phase: bin, sort, count, scan, emit; the pair count ends up in S.off[n].
 cudaError_t pairs_launch(const double *pos, const double *rad, long long n, const Grid &g,
                          double margin, const PairScratch &S, long long cap, int *I, int *J, int *C,
-                         int nsm, cudaStream_t st) {
+                         cudaStream_t st) {
   const long long ncell = (long long)g.B * g.B * g.B;
   cudaMemsetAsync(S.count, 0, sizeof(int) * ncell, st);
   k_bin_q<<<blocks(n), kT, 0, st>>>(pos, rad, n, g, S.key, S.cnt, S.count, S.raw);
   exclusive_scan(S.count, S.start, ncell, S.ws, st);
   k_scatter_q<<<blocks(n), kT, 0, st>>>(n, S.key, S.cnt, S.start, S.tmp);
-  k_place<<<blocks(n), kT, 0, st>>>(n, S.tmp, S.key, S.count, S.start, S.raw, S.order, S.cr);
-  const PairView v{pos, rad, S.order, S.cr, S.count, S.start, margin, n};
+  k_place<<<blocks(n), kT, 0, st>>>(n, S.tmp, S.key, S.start, S.raw, S.order, S.cr);
+  const PairView v{pos, rad, S.order, S.cr, S.start, margin, n};
   const int keep = n <= kPairSlots ? kPairKeep : 0;
-  // cells per warp: several fillings of the chip (64 warps per SM) before a warp takes more
-  int per = 1;
-  while (per < 32 && ncell / per > 256LL * nsm) per *= 2;
-  const long long warps = (ncell + per - 1) / per;
-  k_pair_count<<<blocks(32 * warps), kT, 0, st>>>(v, g, ncell, per, S.list, keep, S.cnt);
+  k_pair_count<<<blocks(n), kT, 0, st>>>(v, g, S.list, keep, S.cnt);
   exclusive_scan(S.cnt, S.off, n, S.ws, st);
   k_pair_emit<<<blocks(n), kT, 0, st>>>(v, g, S.list, keep, S.off, PairOut{cap, I, J, C});
   return cudaGetLastError();
@@ -445,16 +418,6 @@ dem_status read_extent(const double ext[8], double lo[3], double hi[3], double *
   }
   *rmax = ext[6];
   return DEM_OK;
-}
-
-int sm_count() {
-  int dev = 0, v = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1) {
-    cudaGetLastError();
-    return 152;
-  }
-  return v;
 }
 
 // Pinned words that a query's results are copied to, kept between calls (a few per
@@ -567,7 +530,7 @@ extern "C" dem_status dem_find_pairs(const double *pos_dev, const double *radius
   }
   carve_grid(mem2, n, ncell, S);
   const cudaError_t e = pairs_launch(pos_dev, radius_dev, n, g, margin, S, cap, id1_dev, id2_dev,
-                                     cell_dist_dev, sm_count(), st);
+                                     cell_dist_dev, st);
   if (e != cudaSuccess) return done(DEM_ERR_CUDA, std::string("pair query: ") + cudaGetErrorString(e));
   if ((r = fetch(S.off + n, sizeof(int)))) return done(r, err);
   int tot = 0;
@@ -694,7 +657,7 @@ extern "C" dem_status dem_find_pairs_noalloc(const double *pos_dev, const double
   if (!r) r = pair_grid(periodic, cell_h, lo, hi, rmax, margin, g, err, kNoAllocMaxSide);
   if (r) return fail(r, err);
   if (pairs_launch(pos_dev, radius_dev, n, g, margin, S, cap, id1_dev, id2_dev, cell_dist_dev,
-                   sm_count(), st) != cudaSuccess)
+                   st) != cudaSuccess)
     return fail(DEM_ERR_CUDA, "pair query launch failed");
   int tot = 0;
   if ((r = fetch(&tot, S.off + n, sizeof tot))) return fail(r, err);

@@ -207,14 +207,13 @@ struct dem_scene {
   double4_32a *gF = nullptr, *gT = nullptr;
   float4 *wpos = nullptr;
   int4 *cinfo = nullptr;
-  unsigned *cand_list = nullptr;   // the count pass's candidates (kCandKeep per body)
-  int *cand_n = nullptr;
+  unsigned *cand_list = nullptr;   // partners of each body (kCandKeep per body)
 
   Table tab[2]{};
   long long tab_nbody[2]{0, 0};
   int tc = 0;
 
-  int *cell_count = nullptr, *cell_start = nullptr, *cell_fill = nullptr;
+  int *cell_count = nullptr, *cell_start = nullptr;
   long long cell_cap = 0;
   int *scan_ws = nullptr;
   size_t scan_ws_bytes = 0;
@@ -257,6 +256,7 @@ struct dem_scene {
   bool table_fresh = false;   // table rows hold the contacts of the last completed step
   bool check_lost = false;
   bool cs_dirty = true;
+  bool staging_busy = false;  // a copy out of cs_rb may still be under way
   bool layout_dirty = true;      // bodies added or removed since the last collider run
   bool has_walls = false;        // some sub-scene has walls
   bool mixed = false;
@@ -325,7 +325,10 @@ dem_status wait(dem_scene *s) {
   int spins = 0;
   while (true) {
     cudaError_t e = cudaEventQuery(s->ev);
-    if (e == cudaSuccess) return DEM_OK;
+    if (e == cudaSuccess) {
+      s->staging_busy = false;
+      return DEM_OK;
+    }
     if (e != cudaErrorNotReady) return cuda_fail(s, e, "stream wait");
     if (now_s() > deadline) {
       s->broken = true;
@@ -491,12 +494,12 @@ dem_status ensure_bodies(dem_scene *s, long long need) {
   s->slot_of_id = sid;
   dfree(s, s->new_to_old); dfree(s, s->cnt_up); dfree(s, s->cnt_down); dfree(s, s->key);
   dfree(s, s->gF); dfree(s, s->gT); dfree(s, s->wpos); dfree(s, s->cinfo);
-  dfree(s, s->cand_list); dfree(s, s->cand_n);
+  dfree(s, s->cand_list);
   if ((r = dalloc(s, &s->new_to_old, nc)) || (r = dalloc(s, &s->cnt_up, nc)) ||
       (r = dalloc(s, &s->cnt_down, nc)) || (r = dalloc(s, &s->key, nc)) ||
       (r = dalloc(s, &s->gF, nc)) || (r = dalloc(s, &s->gT, nc)) ||
       (r = dalloc(s, &s->wpos, nc)) || (r = dalloc(s, &s->cinfo, nc)) ||
-      (r = dalloc(s, &s->cand_list, nc * kCandKeep)) || (r = dalloc(s, &s->cand_n, nc)))
+      (r = dalloc(s, &s->cand_list, nc * kCandKeep)))
     return r;
   s->cap = nc;
   size_t ws = scan_workspace_bytes(nc + 1);
@@ -563,11 +566,18 @@ dem_status upload_cell(dem_scene *s) {
     cell_derive(u.cs);
     u.cs.dt_law = u.cs.dt;
   }
+  // the staging buffer is rewritten only once its last copy is done (any wait since then);
+  // the read-back into it after a batch is ordered behind the copy on the stream
+  if (s->staging_busy) {
+    const dem_status r = wait(s);
+    if (r) return r;
+  }
   for (int q = 0; q < s->nsub(); ++q) s->cs_rb[q] = s->subs[q].cs;
   CK(cudaMemcpyAsync(s->cs_d, s->cs_rb, sizeof(CellState) * s->nsub(), cudaMemcpyHostToDevice,
                      s->st));
+  s->staging_busy = true;
   s->cs_dirty = false;
-  return wait(s);   // the pinned staging buffer is read again after each batch
+  return DEM_OK;
 }
 
 dem_status status_error(dem_scene *s, int e) {
@@ -583,14 +593,13 @@ dem_status status_error(dem_scene *s, int e) {
 // ------------------------------------------------------------------ collider
 dem_status rebuild_core(dem_scene *s);
 
-// kernels the collider launches (bin, scan x2-3, scatter, cellsort, reorder, count,
-// scans, emit, down sort, degree order x3, merge, lost): counted approximately from
-// its phases
+// kernels the collider launches: bin, scan x2, scatter, reorder, partners, scan x2, rows,
+// downs, degree order, lost (small scans take one launch; a bounding box one more)
 dem_status rebuild(dem_scene *s) {
   if (s->timing) CK(cudaEventRecord(s->tev[0], s->st));
   dem_status r = rebuild_core(s);
   if (r) return r;
-  s->launches += 17 + (s->mixed ? 1 : 0);
+  s->launches += 12;
   if (s->timing) {
     CK(cudaEventRecord(s->tev[1], s->st));
     CK(cudaEventSynchronize(s->tev[1]));
@@ -738,10 +747,8 @@ dem_status rebuild_core(dem_scene *s) {
   for (int q = 0; q < nsub; ++q) s->grids_h[q] = s->subs[q].grid;
   CK(cudaMemcpyAsync(s->grids_d, s->grids_h, sizeof(Grid) * nsub, cudaMemcpyHostToDevice, s->st));
   if (ncell > s->cell_cap) {
-    dfree(s, s->cell_count); dfree(s, s->cell_start); dfree(s, s->cell_fill);
-    if ((r = dalloc(s, &s->cell_count, ncell)) || (r = dalloc(s, &s->cell_start, ncell + 1)) ||
-        (r = dalloc(s, &s->cell_fill, ncell)))
-      return r;
+    dfree(s, s->cell_count); dfree(s, s->cell_start);
+    if ((r = dalloc(s, &s->cell_count, ncell)) || (r = dalloc(s, &s->cell_start, ncell + 1))) return r;
     s->cell_cap = ncell;
     size_t ws = scan_workspace_bytes(ncell + 1);
     if (ws > s->scan_ws_bytes) {
@@ -751,7 +758,6 @@ dem_status rebuild_core(dem_scene *s) {
     }
   }
   CK(cudaMemsetAsync(s->cell_count, 0, sizeof(int) * ncell, s->st));
-  CK(cudaMemsetAsync(s->cell_fill, 0, sizeof(int) * ncell, s->st));
   CK(cudaMemsetAsync(&s->ds_d->error, 0, sizeof(int), s->st));
   // ids close up over removed sub-scenes: each live sub-scene's ids move down by the
   // bodies of removed sub-scenes with smaller ids
@@ -767,32 +773,29 @@ dem_status rebuild_core(dem_scene *s) {
                        s->st));
     id_shift = s->id_shift_d;
   }
-  // 2-3: bin, counting sort (cell order, then id within a cell), permute the bodies
-  launch_bin(s->cur, N, s->grids_d, multi, dead, s->key, s->cell_count, s->st);
+  // 2-3: bin, counting sort (cell order, then id within a cell), permute the bodies and
+  // their records.  Scratch: the up / down counts hold the arrival order and places until
+  // the walk writes them, the force buffer (used by queries only) the unsorted records.
+  const CellRec raw{reinterpret_cast<float4 *>(s->gF), reinterpret_cast<int4 *>(s->gF) + s->cap};
+  const CellRec cr{s->wpos, s->cinfo};
+  int *tmp = s->cnt_up, *rank = s->cnt_down;
+  launch_bin(s->cur, N, s->grids_d, multi, dead, s->key, rank, s->cell_count, raw, s->st);
   exclusive_scan(s->cell_count, s->cell_start, ncell, s->scan_ws, s->st);
-  launch_scatter(N, s->key, s->cell_start, s->cell_fill, s->new_to_old, s->st);
-  // the sentinel cell of removed bodies is left unsorted: its order is never used (and
-  // it can hold every body of a large removed sub-scene)
-  launch_cellsort(s->cell_count, s->cell_start, total, s->cur.id, s->new_to_old, s->st);
-  launch_reorder(s->cur, s->alt, n_live, s->cap, s->new_to_old, s->slot_of_id, s->has_walls,
-                 s->mixed, id_shift, s->st);
+  launch_scatter(N, s->key, rank, s->cell_start, tmp, s->st);
+  launch_reorder(s->cur, s->alt, n_live, s->cap, tmp, s->key, s->cell_start, raw, cr, s->new_to_old,
+                 s->slot_of_id, s->has_walls, s->mixed, id_shift, s->st);
   std::swap(s->cur, s->alt);
-  const long long N_old = N;
   s->N = n_live;
   const long long NL = n_live;
-  // 4: candidates (count, prefix sums, emit)
+  // 4: partners of every body, prefix sums of the two counts
   Table &ot = s->tab[s->tc];
   Table &nt = s->tab[1 - s->tc];
   if ((r = ensure_table(s, nt, 0, NL))) return r;
-  launch_cellrec(s->cur, NL, s->grids_d, multi, s->wpos, s->cinfo, s->st);
-  CK(cudaMemsetAsync(s->cnt_up, 0, sizeof(int) * std::max<long long>(NL, 1), s->st));
-  CK(cudaMemsetAsync(s->cnt_down, 0, sizeof(int) * std::max<long long>(NL, 1), s->st));
-  // slots are packed in 26 bits of a candidate entry
-  const CandList cl{s->cand_list, s->cand_n, s->cap < (1LL << 26) ? 1 : 0};
-  launch_count(s->wpos, s->cinfo, s->cur.sid, s->cur.id, NL, s->grids_d, multi, s->cell_count,
-               s->cell_start, s->cnt_up, s->cnt_down, &s->ds_d->error, cl, s->st);
-  exclusive_scan(s->cnt_up, nt.row_start, NL, s->scan_ws, s->st);
-  exclusive_scan(s->cnt_down, nt.down_start, NL, s->scan_ws, s->st);
+  // slots are packed in 26 bits of a list entry
+  const CandList cl{s->cand_list, s->cap < (1LL << 26) ? kCandKeep : 0};
+  launch_partners(cr, s->cur.sid, s->cur.id, NL, s->grids_d, multi, s->cell_start, s->cnt_up,
+                  s->cnt_down, &s->ds_d->error, cl, s->st);
+  exclusive_scan2(s->cnt_up, nt.row_start, s->cnt_down, nt.down_start, NL, s->scan_ws, s->st);
   CK(cudaMemcpyAsync(&s->rb_h->totals[0], nt.row_start + NL, sizeof(int), cudaMemcpyDeviceToHost, s->st));
   CK(cudaMemcpyAsync(&s->rb_h->totals[1], nt.down_start + NL, sizeof(int), cudaMemcpyDeviceToHost, s->st));
   CK(cudaMemcpyAsync(&s->rb_h->ds, s->ds_d, sizeof(DevStatus), cudaMemcpyDeviceToHost, s->st));
@@ -802,27 +805,17 @@ dem_status rebuild_core(dem_scene *s) {
   if (P != s->rb_h->totals[1]) return fail(s, DEM_ERR_STATE, "internal: candidate count mismatch");
   if ((r = ensure_table(s, nt, P, NL))) return r;
   nt.P = P;
-  // fill counters: the bin keys and the up counts (scanned already) are no longer needed
-  int *dfill = reinterpret_cast<int *>(s->key);
-  int *ufill = s->cnt_up;
-  CK(cudaMemsetAsync(dfill, 0, sizeof(int) * std::max<long long>(NL, 1), s->st));
-  CK(cudaMemsetAsync(ufill, 0, sizeof(int) * std::max<long long>(NL, 1), s->st));
-  launch_emit(s->wpos, s->cinfo, s->cur, NL, s->grids_d, multi, s->cell_count, s->cell_start, nt,
-              ufill, dfill, cl, s->st);
-  if (s->mixed) launch_ref_branch(nt, s->cur, s->grids_d, multi, s->st);
-  launch_downsort(nt, s->cur.id, NL, s->st);
-  CK(cudaMemsetAsync(s->deg_ws, 0, sizeof(int) * 2 * kDegreeBuckets, s->st));
-  launch_degree_order(nt, NL, s->deg_ws, s->st);
-  // 5: carry the contact history of the previous table
+  // 5-6: rows with the contact history of the previous table, down lists
   ot.P = std::min(ot.P, ot.cap);
   if (ot.P > 0) CK(cudaMemsetAsync(ot.found, 0, sizeof(int) * ot.P, s->st));
   Table otv = ot;
   if (ot.P == 0 || ot.row_start == nullptr) otv.P = 0;
-  launch_merge(nt, otv, s->tab_nbody[s->tc], s->new_to_old, s->mixed, s->st);
+  launch_rows(cr, s->cur, s->grids_d, multi, s->cell_start, nt, otv, NL,
+              s->tab_nbody[s->tc], s->new_to_old, cl, s->mixed, s->st);
+  launch_degree_order(nt, NL, s->st);
   // a removed sub-scene's contacts vanish by design: no history check on that run
   if (s->check_lost && !removal)
     launch_lost(otv, s->alt, s->grids_d, multi, &s->ds_d->error, s->mixed, s->st);
-  (void)N_old;
   s->tab_nbody[1 - s->tc] = NL;
   s->tc = 1 - s->tc;
   // host bookkeeping of removals: ids and per-id host arrays close up
@@ -906,7 +899,7 @@ double scene_bytes_per_body(int mixed) {
   double buf = 6 * d4 + 3 * sizeof(int) + sizeof(uint8_t) + sizeof(double) + 6 * d4;
   if (mixed) buf += 6 * f4;
   const double scratch = 5 * sizeof(int) + 2 * d4 + f4 + sizeof(int4) +
-                        kCandKeep * sizeof(unsigned) + sizeof(int);
+                        kCandKeep * sizeof(unsigned);
   const double tables = 2 * 3 * sizeof(int);
   return 2 * buf + scratch + tables;
 }
@@ -1071,8 +1064,8 @@ void dem_scene_destroy(dem_scene *s) {
   free_table(s, s->tab[1]);
   dfree(s, s->slot_of_id); dfree(s, s->new_to_old); dfree(s, s->cnt_up); dfree(s, s->cnt_down);
   dfree(s, s->key); dfree(s, s->gF); dfree(s, s->gT); dfree(s, s->wpos); dfree(s, s->cinfo);
-  dfree(s, s->cand_list); dfree(s, s->cand_n);
-  dfree(s, s->cell_count); dfree(s, s->cell_start); dfree(s, s->cell_fill);
+  dfree(s, s->cand_list);
+  dfree(s, s->cell_count); dfree(s, s->cell_start);
   dfree(s, s->scan_ws); dfree(s, s->partials); dfree(s, s->servo); dfree(s, s->p3d_d); dfree(s, s->p3d_part); dfree(s, s->deg_ws);
   dfree(s, s->mats_d); dfree(s, s->cs_d); dfree(s, s->ds_d);
   dfree(s, s->grids_d); dfree(s, s->id_shift_d); dfree(s, s->bbox_keys); dfree(s, s->dt_keys);
