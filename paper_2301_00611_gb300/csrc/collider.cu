@@ -157,7 +157,8 @@ __global__ void k_reorder(Bodies src, Bodies dst, long long N, long long cap,
                           const int *__restrict__ tmp, const uint32_t *__restrict__ key,
                           const int *__restrict__ start, CellRec raw,
                           CellRec cr, int *new_to_old, int *slot_of_id, int has_walls, int mixed,
-                          const int *__restrict__ id_shift) {
+                          const int *__restrict__ id_shift, const CellState *__restrict__ cs,
+                          int multi) {
   const long long at = (long long)blockIdx.x * kT + threadIdx.x;
   if (at >= N) return;
   const int o = tmp[at];
@@ -195,9 +196,25 @@ __global__ void k_reorder(Bodies src, Bodies dst, long long N, long long cap,
   const uint8_t flags = src.flags[o];
   dst.flags[p] = flags;
   slot_of_id[id] = p;
-  if (has_walls)   // a wall history is read only while its flag is set
-    for (int w = 0; w < 6; ++w)
+  dst.live[p] = 0;
+  uint8_t near = 0;
+  if (has_walls) {
+    // a body moves at most the sweep margin from x before the next run, so it can only meet
+    // the walls within r + margin now (FP32 distances, with room for their rounding)
+    const CellState &c = cs[multi ? q : 0];
+    const float reach = (float)(x.w + c.verlet) * 1.0001f;
+    const double xs[3] = {x.x, x.y, x.z};
+    for (int w = 0; w < 6; ++w) {
+      if (c.wall_mask & (1 << w)) {
+        const int ax = w >> 1;
+        const float d = (float)(xs[ax] - ((w & 1) ? c.box_hi[ax] : c.box_lo[ax]));
+        if (!(fabsf(d) * 0.9999f > reach)) near |= (uint8_t)(1 << w);
+      }
+      // a wall history is read only while its flag is set
       if (flags & (2 << w)) dst.whist[w * cap + p] = src.whist[w * cap + o];
+    }
+  }
+  dst.wnear[p] = near;
 }
 
 // Does the shift of j seen from s leave the range of a packed shift?
@@ -635,10 +652,10 @@ void launch_scatter(long long N, const uint32_t *key, const int *rank, const int
 void launch_reorder(const Bodies &src, const Bodies &dst, long long N, long long cap,
                     const int *tmp, const uint32_t *key, const int *start, CellRec raw, CellRec cr,
                     int *new_to_old, int *slot_of_id, int has_walls,
-                    int mixed, const int *id_shift, cudaStream_t st) {
+                    int mixed, const int *id_shift, const CellState *cs, int multi, cudaStream_t st) {
   if (N > 0)
     k_reorder<<<blocks(N), kT, 0, st>>>(src, dst, N, cap, tmp, key, start, raw, cr,
-                                        new_to_old, slot_of_id, has_walls, mixed, id_shift);
+                                        new_to_old, slot_of_id, has_walls, mixed, id_shift, cs, multi);
 }
 
 void launch_partners(CellRec cr, const int *sid, const int *id, long long N, const Grid *grids,

@@ -161,6 +161,8 @@ __device__ __forceinline__ void real_row_mixed(const Table &t, const Bodies &b,
   }
   const float Fx = Fn * nx + sx, Fy = Fn * ny + sy, Fz = Fn * nz + sz;
   const float d1 = r1 - 0.5f * pen, d2 = r2 - 0.5f * pen;
+  b.live[pr.x] = 1;
+  b.live[pr.y] = 1;
   t.hfs[k] = make_double4_32a(fx, fy, fz, tanphi);
   t.hn32[k] = make_float4(nx, ny, nz, ks);
   t.oFM32[2 * k] = make_float4(Fx, Fy, Fz, d1);
@@ -169,13 +171,15 @@ __device__ __forceinline__ void real_row_mixed(const Table &t, const Bodies &b,
 
 // Same per-warp queue of real rows as the FP64 kernel: the FP32 geometry test on
 // tiles of 32 consecutive rows, the law on 32 queued real rows at a time.
+// 64 registers: half of the SM's warps, which the kernel's scattered loads need (at 80
+// registers, three eighths of the warps, 1M dense spheres took 171 us instead of 148).
 template <int kT, int kFeat, bool kDesc>
-__global__ void __launch_bounds__(kT) k_contact_mixed(const StepDesc *__restrict__ d,
+__global__ void __launch_bounds__(kT, 1024 / kT) k_contact_mixed(const StepDesc *__restrict__ d,
                                                       Table tp, Bodies bp,
                                                       const CellState *__restrict__ cs,
                                                       const DevStatus *__restrict__ ds,
                                                       const Mat *__restrict__ mats, int multi) {
-  constexpr int kWarps = kT / 32;
+  constexpr int kWarps = kT / 32;   // warps of the largest block
   const Table &t = kDesc ? d->t : tp;
   const Bodies &b = kDesc ? d->b : bp;
   if (ds->pending) return;
@@ -184,9 +188,9 @@ __global__ void __launch_bounds__(kT) k_contact_mixed(const StepDesc *__restrict
   QRowF *wq = q[wi];
   const RowCellF rc0 = row_cell_f(cs[0]);
   const long long P = t.P;
-  const long long stride = (long long)gridDim.x * kT;
+  const long long stride = (long long)gridDim.x * blockDim.x;
   int cnt = 0;
-  for (long long base = (long long)blockIdx.x * kT + wi * 32; base < P; base += stride) {
+  for (long long base = (long long)blockIdx.x * blockDim.x + wi * 32; base < P; base += stride) {
     const long long k = base + lane;
     bool real = false;
     float dx = 0, dy = 0, dz = 0, l2 = 0, r1 = 0, r2 = 0, gap2 = 0;
@@ -236,6 +240,7 @@ __global__ void __launch_bounds__(kT) k_contact_mixed(const StepDesc *__restrict
       }
     }
     const unsigned m = __ballot_sync(0xffffffffu, real);
+    if (lane == 0) t.bits[base >> 5] = m;
     if (real) {
       const int at = cnt + __popc(m & ((1u << lane) - 1u));
       wq[at] = QRowF{dx, dy, dz, l2, r1, r2, k, sq, gap2};
@@ -262,11 +267,18 @@ void launch_contact_mixed(const StepDesc *d, const StepDesc &h, bool desc, long 
                           const CellState *cs, const DevStatus *ds, const Mat *mats, int multi,
                           int feat, int nsm, int block, int per_sm, cudaStream_t st) {
   if (rows <= 0) return;
+  const int regs = block;   // which register budget: that of the tuned block
+  block = spread_block(rows, block, nsm);
   long long need = (rows + block - 1) / block;
-  long long cap = (long long)nsm * per_sm;   // persistent grid: per_sm blocks per SM
+  // Persistent grid: at most the blocks an SM holds at a time.  Further ones repeat the
+  // start-up and end with a partly filled pass of the law for each of their warps: four
+  // blocks of 256 an SM instead of eight, 1M dense spheres 148 -> 140 us, 789k in 64 loose
+  // scenes 45 -> 40 (three an SM: 163 and 45).
+  const int resident = 1024 / block;
+  const long long cap = (long long)nsm * (per_sm < resident ? per_sm : resident);
   unsigned grid = (unsigned)(need < cap ? need : cap);
-#define DEM_C(B, F, D) k_contact_mixed<B, F, D><<<grid, B, 0, st>>>(d, h.t, h.b, cs, ds, mats, multi)
-#define DEM_CB(F, D) if (block == 128) DEM_C(128, F, D); else DEM_C(256, F, D);
+#define DEM_C(B, F, D) k_contact_mixed<B, F, D><<<grid, block, 0, st>>>(d, h.t, h.b, cs, ds, mats, multi)
+#define DEM_CB(F, D) if (regs == 128 && block == 128) DEM_C(128, F, D); else DEM_C(256, F, D);
 #define DEM_CF(D) switch (feat & 3) { case 0: DEM_CB(0, D) break; case 1: DEM_CB(1, D) break; \
                                       case 2: DEM_CB(2, D) break; default: DEM_CB(3, D) }
   if (desc) { DEM_CF(true) } else { DEM_CF(false) }

@@ -73,6 +73,9 @@ struct Bodies {
   int *id, *mat;
   int *sid;         // sub-scene of each body (read only when SceneConst::multi)
   uint8_t *flags;   // bit0 fixed; bit (1+w) in contact with wall w
+  uint8_t *live;    // 1: a real row touched the body since its last integration (the contact
+                    // kernel sets it, the integrator reads and clears it)
+  uint8_t *wnear;   // bit w: the body can reach wall w before the next collider run
   double4_32a *whist;   // [6 * cap] or null
   double *rdsc;     // 1 / density-scaling factor of each body (1: unscaled)
   // mixed precision mirrors (null in FP64 mode), written by the integrator:
@@ -89,6 +92,7 @@ struct Table {
   double4_32a *hfs, *hn;   // FP64 mode; mixed mode uses hfs = (Fs, tan(phi))
   double4_32a *oFM;        // [2 * rows]: (F on body 2, d1), (-(n x F), d2) per row
   double *tanphi;
+  unsigned *bits;   // bit k % 32 of word k / 32: row k is real in the current step
   // mixed precision rows (null in FP64 mode)
   float4 *g32;      // (reference branch vector xref2 + Href c - xref1, kn); kn == 0: not real
   float *s0;        // (r1 + r2)^2 - |reference branch vector|^2, formed in FP64 at the
@@ -275,7 +279,7 @@ void launch_scatter(long long N, const uint32_t *key, const int *rank, const int
 void launch_reorder(const Bodies &src, const Bodies &dst, long long N, long long cap,
                     const int *tmp, const uint32_t *key, const int *start, CellRec raw, CellRec cr,
                     int *new_to_old, int *slot_of_id, int has_walls, int mixed,
-                    const int *id_shift, cudaStream_t st);
+                    const int *id_shift, const CellState *cs, int multi, cudaStream_t st);
 // per-sub-scene bounding boxes as ordered keys (see collider.cu); keys preset
 void launch_bbox_sub(const Bodies &b, long long N, int cap, unsigned long long *keys, int nsm,
                      cudaStream_t st);
@@ -323,11 +327,23 @@ void launch_contact_mixed(const StepDesc *d, const StepDesc &h, bool desc, long 
                           const CellState *cs, const DevStatus *ds, const Mat *mats, int multi,
                           int feat, int nsm, int block, int per_sm, cudaStream_t st);
 
+// Block size of a step kernel over n rows or bodies: the tuned one, unless its blocks leave
+// SMs idle -- then the largest of 128, 64, 32 that makes at least four blocks an SM.  In a
+// small scene a step is the time of its slowest SM, and eight warps that share one SM's FP64
+// pipe wait for one another: 1000 spheres in a walled box, integration 20.6 -> 16.6 us in
+// blocks of 32 instead of 256.
+inline int spread_block(long long n, int tuned, int nsm) {
+  int b = tuned;
+  while (b > 32 && n < 4LL * nsm * b) b = b > 128 ? 128 : b / 2;
+  return b;
+}
+
 // integrate.cu
 // block: 128, 256 or 512 threads
 // h.sc.N and h.sc.walls size and select the launch (and must match *d when desc)
 void launch_integrate(const StepDesc *d, const StepDesc &h, bool desc, const CellState *cs,
-                      DevStatus *ds, const Mat *mats, int mixed, int block, cudaStream_t st);
+                      DevStatus *ds, const Mat *mats, int mixed, int block, int nsm,
+                      cudaStream_t st);
 // one thread per sub-scene (cs[0 .. nsub)); servo partials apply to sub-scene 0
 void launch_cell_advance(CellState *cs, int nsub, DevStatus *ds, const double *servo_partials,
                          cudaStream_t st, P3d *p3d = nullptr, const double *p3d_partials = nullptr);

@@ -104,6 +104,93 @@ __device__ inline void gather_rows_f32(const Table &t, int s, float F[3], float 
   T[0] = t0; T[1] = t1; T[2] = t2;
 }
 
+// The same sums over the real rows only, for the step kernels: a row that is not in
+// contact adds an exact zero, so leaving it out changes no bit.  A quarter (loose clouds:
+// nearly all) to a half of a table's rows are not, and each cost its two readers a scattered
+// record and, in FP64, twelve instructions of the FP64 pipe.  The contact kernel leaves one
+// bit a row; a body's bits over its concatenated lists (own rows: a shifted word, down
+// rows: a gather of bits that sit in cache) make a mask, 32 rows at a time, whose set bits
+// are walked two at a time; a body that no real row touched (its flag) skips the lists.
+// FP64, 300k loose spheres 96 -> 77 us, 1M dense 330 -> 307; mixed, 789k spheres in 64 walled
+// scenes 155 -> 104 us (with the walls out of reach skipped and 64 registers).
+struct RowList {
+  int e0, nd, r0, n;   // down entries [e0, e0 + nd), then rows r0 + j for j in [nd, n)
+};
+__device__ inline RowList row_list(const Table &t, int s) {
+  RowList l;
+  l.e0 = t.down_start[s];
+  l.nd = t.down_start[s + 1] - l.e0;
+  const int a = t.row_start[s];
+  l.r0 = a - l.nd;
+  l.n = l.nd + (t.row_start[s + 1] - a);
+  return l;
+}
+__device__ inline unsigned real_mask(const Table &t, const RowList &l, int j0) {
+  const int end = min(l.n, j0 + 32), dn = min(l.nd, j0 + 32);
+  unsigned m = 0;
+  if (end > l.nd) {   // own rows: consecutive bits
+    const int p = max(l.nd, j0), a = l.r0 + p, cnt = end - p;
+    const unsigned w = __funnelshift_r(t.bits[a >> 5], t.bits[(a >> 5) + 1], a & 31);
+    m = (w & (0xffffffffu >> (32 - cnt))) << (p - j0);
+  }
+#pragma unroll 4
+  for (int j = j0; j < dn; ++j) {
+    const int k = t.down[l.e0 + j];
+    m |= ((t.bits[k >> 5] >> (k & 31)) & 1u) << (j - j0);
+  }
+  return m;
+}
+
+__device__ inline void gather_real(const Table &t, const RowList &l, double F[3], double T[3]) {
+  for (int j0 = 0; j0 < l.n; j0 += 32) {
+    unsigned m = real_mask(t, l, j0);
+    while (m) {
+      const int ja = j0 + __ffs(m) - 1;
+      m &= m - 1;
+      const bool two = m != 0;
+      const int jb = two ? j0 + __ffs(m) - 1 : ja;
+      m &= m - 1;
+      const bool a1 = ja >= l.nd, b1 = jb >= l.nd;   // body 1 of the row
+      const long long ka = a1 ? l.r0 + ja : t.down[l.e0 + ja];
+      const long long kb = b1 ? l.r0 + jb : t.down[l.e0 + jb];
+      const double4_32a fa = t.oFM[2 * ka], ma = t.oFM[2 * ka + 1], fb = t.oFM[2 * kb], mb = t.oFM[2 * kb + 1];
+      const double sa = a1 ? -1.0 : 1.0, da = a1 ? fa.w : ma.w;
+      F[0] += sa * fa.x; F[1] += sa * fa.y; F[2] += sa * fa.z;
+      T[0] += da * ma.x; T[1] += da * ma.y; T[2] += da * ma.z;
+      if (two) {
+        const double sb = b1 ? -1.0 : 1.0, db = b1 ? fb.w : mb.w;
+        F[0] += sb * fb.x; F[1] += sb * fb.y; F[2] += sb * fb.z;
+        T[0] += db * mb.x; T[1] += db * mb.y; T[2] += db * mb.z;
+      }
+    }
+  }
+}
+
+__device__ inline void gather_real_f32(const Table &t, const RowList &l, float F[3], float T[3]) {
+  for (int j0 = 0; j0 < l.n; j0 += 32) {
+    unsigned m = real_mask(t, l, j0);
+    while (m) {
+      const int ja = j0 + __ffs(m) - 1;
+      m &= m - 1;
+      const bool two = m != 0;
+      const int jb = two ? j0 + __ffs(m) - 1 : ja;
+      m &= m - 1;
+      const bool a1 = ja >= l.nd, b1 = jb >= l.nd;
+      const long long ka = a1 ? l.r0 + ja : t.down[l.e0 + ja];
+      const long long kb = b1 ? l.r0 + jb : t.down[l.e0 + jb];
+      const float4 fa = t.oFM32[2 * ka], ma = t.oFM32[2 * ka + 1], fb = t.oFM32[2 * kb], mb = t.oFM32[2 * kb + 1];
+      const float sa = a1 ? -1.0f : 1.0f, da = a1 ? fa.w : ma.w;
+      F[0] += sa * fa.x; F[1] += sa * fa.y; F[2] += sa * fa.z;
+      T[0] += da * ma.x; T[1] += da * ma.y; T[2] += da * ma.z;
+      if (two) {
+        const float sb = b1 ? -1.0f : 1.0f, db = b1 ? fb.w : mb.w;
+        F[0] += sb * fb.x; F[1] += sb * fb.y; F[2] += sb * fb.z;
+        T[0] += db * mb.x; T[1] += db * mb.y; T[2] += db * mb.z;
+      }
+    }
+  }
+}
+
 // Physics of a sphere-wall contact: FrictPhys with equivalent wall radius = sphere
 // radius, or (law 1) the Hertz-Mindlin constants with an infinite wall radius; wall
 // material = the scene's wall material (material 0 by default).
@@ -121,6 +208,11 @@ __device__ inline void wall_phys(const Mat *mats, int wmat, int mat, double r, d
   ks = s1 * s2 / (s1 + s2);
 }
 
+template <class T>
+__device__ __forceinline__ T pick(int k, T a, T b, T c) {
+  return k == 0 ? a : (k == 1 ? b : c);
+}
+
 // Mixed precision integrator: FP32 force sum, walls, damping and orientation;
 // FP64 only where the velocity and position accumulate (v += dv, x += dt v) and in
 // the offset of the new position from its reference (rounded once to FP32 for the
@@ -129,8 +221,10 @@ __device__ inline void wall_phys(const Mat *mats, int wmat, int mat, double r, d
 // instructions per body.
 // kFeat: bit 0 some sub-scene has walls, bit 1 some periodic cell is sheared (full 3x3
 // products); each variant carries only the branches it needs.
-template <int kB, int kFeat, bool kDesc>
-__global__ void __launch_bounds__(kB) k_integrate_mixed(const StepDesc *__restrict__ d, StepDesc hp,
+// Registers: 64 where the wall law is compiled in (two blocks of 512, half of the SM's
+// warps; its spills sit on the path of the few bodies at a wall), as needed elsewhere.
+template <int kFeat, bool kDesc>
+__global__ void __launch_bounds__(512, (kFeat & 1) ? 2 : 3) k_integrate_mixed(const StepDesc *__restrict__ d, StepDesc hp,
                                                         const CellState *__restrict__ cs,
                                                         DevStatus *ds, const Mat *__restrict__ mats) {
   if (ds->pending) return;
@@ -138,14 +232,18 @@ __global__ void __launch_bounds__(kB) k_integrate_mixed(const StepDesc *__restri
   const Table &t = kDesc ? d->t : hp.t;
   const SceneConst &sc = kDesc ? d->sc : hp.sc;
   const long long cap = kDesc ? d->cap : hp.cap;
-  const long long sl = (long long)blockIdx.x * kB + threadIdx.x;
+  const long long sl = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (sl >= sc.N) return;
   const int s = sc.ordered ? t.ord[sl] : (int)sl;
   const CellState &c = cs[sc.multi ? b.sid[s] : 0];
   const double dt = c.dt;
   const float dtf = (float)dt;
-  float F[3], T[3];
-  gather_rows_f32(t, s, F, T);   // fixed order, FP32 sums
+  float F[3] = {0, 0, 0}, T[3] = {0, 0, 0};
+  const RowList rows = row_list(t, s);   // (loaded beside the flag, not after it)
+  if (b.live[s]) {   // no row of the body is real otherwise
+    b.live[s] = 0;
+    gather_real_f32(t, rows, F, T);   // fixed order, FP32 sums
+  }
   const float4 va = b.vw32[2 * s], vb = b.vw32[2 * s + 1];   // v-, w- in FP32
   const float4 off = b.p32[s];                                // x - xref, r
   const float4 xr = b.xref32[s];
@@ -155,14 +253,17 @@ __global__ void __launch_bounds__(kB) k_integrate_mixed(const StepDesc *__restri
   const float xf[3] = {xr.x + off.x, xr.y + off.y, xr.z + off.z};
   const float r = off.w;
 
-  if ((kFeat & 1) && c.wall_mask) {   // sphere-wall contacts: the FP64 kernel's law, in FP32
+  // sphere-wall contacts: the FP64 kernel's law, in FP32; only the walls within reach, or
+  // in contact, are looked at
+  const int walls = (kFeat & 1) ? (b.wnear[s] | ((flags >> 1) & 0x3f)) & c.wall_mask : 0;
+  if ((kFeat & 1) && walls) {
     const float dtl = (float)c.dt_law;   // the contact law's step (see CellState::dt_law)
     const double4_32a pd = b.pos[s];
-    const double xd[3] = {pd.x, pd.y, pd.z};
-    for (int wi = 0; wi < 6; ++wi) {
-      if (!(c.wall_mask & (1 << wi))) continue;
-      const int ax = wi >> 1;
-      const double distd = xd[ax] - ((wi & 1) ? c.box_hi[ax] : c.box_lo[ax]);
+    double knd, ksd, tpd;
+    wall_phys(mats, c.wall_mat, b.mat[s], (double)r, knd, ksd, tpd, c.law);
+    for (int left = walls; left; left &= left - 1) {   // each lane its own walls, in order
+      const int wi = __ffs(left) - 1, ax = wi >> 1;
+      const double distd = pick(ax, pd.x, pd.y, pd.z) - ((wi & 1) ? c.box_hi[ax] : c.box_lo[ax]);
       const float dist = (float)distd;
       const bool was = flags & (2 << wi);
       if (!(fabsf(dist) < r)) {
@@ -173,13 +274,10 @@ __global__ void __launch_bounds__(kB) k_integrate_mixed(const StepDesc *__restri
         continue;
       }
       const float sn = dist >= 0 ? 1.0f : -1.0f;
-      float n[3] = {0, 0, 0};
-      n[ax] = sn;
+      const float n[3] = {ax == 0 ? sn : 0.0f, ax == 1 ? sn : 0.0f, ax == 2 ? sn : 0.0f};
       // the penetration in FP64 and rounded once: r - |dist| in FP32 would keep the
       // precision of r, not of the (much smaller) penetration
       const float pen = (float)(pd.w - fabs(distd));   // FP64 radius and distance
-      double knd, ksd, tpd;
-      wall_phys(mats, c.wall_mat, b.mat[s], (double)r, knd, ksd, tpd, c.law);
       const float sqp = c.law ? sqrtf(pen) : 1.0f;   // Hertz-Mindlin: pen^1/2 factors
       const float kn = (float)knd * sqp, ks = (float)ksd * sqp, tanphi = (float)tpd;
       float fs[3] = {0, 0, 0};
@@ -187,7 +285,7 @@ __global__ void __launch_bounds__(kB) k_integrate_mixed(const StepDesc *__restri
         const double4_32a h = b.whist[wi * cap + s];
         fs[0] = (float)h.x; fs[1] = (float)h.y; fs[2] = (float)h.z;
       }
-      const float tw = 0.5f * dtl * (sn * ww[ax]);
+      const float tw = 0.5f * dtl * (sn * pick(ax, ww[0], ww[1], ww[2]));
       const float tn[3] = {tw * n[0], tw * n[1], tw * n[2]};
       const float c0 = fs[1] * tn[2] - fs[2] * tn[1];
       const float c1 = fs[2] * tn[0] - fs[0] * tn[2];
@@ -320,8 +418,8 @@ __global__ void __launch_bounds__(kB) k_integrate_mixed(const StepDesc *__restri
     atomicOr(&ds->error, kErrNonFinite);
 }
 
-template <int kB, int kFeat, bool kDesc>
-__global__ void __launch_bounds__(kB) k_integrate(const StepDesc *__restrict__ d, StepDesc hp,
+template <int kFeat, bool kDesc>
+__global__ void __launch_bounds__(512) k_integrate(const StepDesc *__restrict__ d, StepDesc hp,
                                                   const CellState *__restrict__ cs,
                                                   DevStatus *ds, const Mat *__restrict__ mats) {
   if (ds->pending) return;
@@ -329,13 +427,17 @@ __global__ void __launch_bounds__(kB) k_integrate(const StepDesc *__restrict__ d
   const Table &t = kDesc ? d->t : hp.t;
   const SceneConst &sc = kDesc ? d->sc : hp.sc;
   const long long cap = kDesc ? d->cap : hp.cap;
-  const long long sl = (long long)blockIdx.x * kB + threadIdx.x;
+  const long long sl = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (sl >= sc.N) return;
   const int s = sc.ordered ? t.ord[sl] : (int)sl;
   const CellState &c = cs[sc.multi ? b.sid[s] : 0];
   const double dt = c.dt;
   double F[3] = {0, 0, 0}, T[3] = {0, 0, 0};
-  gather_rows(t, s, F, T);
+  const RowList rows = row_list(t, s);   // (loaded beside the flag, not after it)
+  if (b.live[s]) {   // no row of the body is real otherwise
+    b.live[s] = 0;
+    gather_real(t, rows, F, T);
+  }
 
   const double4_32a p = b.pos[s];
   const double4_32a v = b.vel[s];
@@ -345,12 +447,14 @@ __global__ void __launch_bounds__(kB) k_integrate(const StepDesc *__restrict__ d
   const double x[3] = {p.x, p.y, p.z}, vv[3] = {v.x, v.y, v.z}, ww[3] = {w.x, w.y, w.z};
   const double r = p.w;
 
-  if ((kFeat & 1) && c.wall_mask) {
-    for (int wi = 0; wi < 6; ++wi) {
-      if (!(c.wall_mask & (1 << wi))) continue;
-      const int ax = wi >> 1;
+  const int walls = (kFeat & 1) ? (b.wnear[s] | ((flags >> 1) & 0x3f)) & c.wall_mask : 0;
+  if ((kFeat & 1) && walls) {   // only the walls within reach or in contact
+    double kn0, ks0, tanphi;
+    wall_phys(mats, c.wall_mat, b.mat[s], r, kn0, ks0, tanphi, c.law);
+    for (int left = walls; left; left &= left - 1) {   // each lane its own walls, in order
+      const int wi = __ffs(left) - 1, ax = wi >> 1;
       const double wc = (wi & 1) ? c.box_hi[ax] : c.box_lo[ax];
-      const double dist = x[ax] - wc;
+      const double dist = pick(ax, x[0], x[1], x[2]) - wc;
       const bool was = flags & (2 << wi);
       if (!(fabs(dist) < r)) {
         if (was) {
@@ -360,11 +464,9 @@ __global__ void __launch_bounds__(kB) k_integrate(const StepDesc *__restrict__ d
         continue;
       }
       const double sn = dist >= 0 ? 1.0 : -1.0;
-      double n[3] = {0, 0, 0};
-      n[ax] = sn;
+      const double n[3] = {ax == 0 ? sn : 0.0, ax == 1 ? sn : 0.0, ax == 2 ? sn : 0.0};
       const double pen = r - fabs(dist);
-      double kn, ks, tanphi;
-      wall_phys(mats, c.wall_mat, b.mat[s], r, kn, ks, tanphi, c.law);
+      double kn = kn0, ks = ks0;
       if (c.law) {   // Hertz-Mindlin: Fn = kno pen^3/2, ks = kso pen^1/2
         const double sq = sqrt(pen);
         kn *= sq;
@@ -377,7 +479,7 @@ __global__ void __launch_bounds__(kB) k_integrate(const StepDesc *__restrict__ d
       }
       // frame motion: n- x n = 0 (the normal is fixed); twist dt/2 n.(0 + w), with the
       // contact law's step (see CellState::dt_law)
-      const double tw = 0.5 * c.dt_law * (sn * ww[ax]);
+      const double tw = 0.5 * c.dt_law * (sn * pick(ax, ww[0], ww[1], ww[2]));
       const double tn[3] = {tw * n[0], tw * n[1], tw * n[2]};
       const double c0 = fs[1] * tn[2] - fs[2] * tn[1];
       const double c1 = fs[2] * tn[0] - fs[0] * tn[2];
@@ -767,8 +869,87 @@ __device__ bool p3d_update(P3d &P, const double *part, const double (&Hp)[9],
   return true;
 }
 
-// Advance of one (sub-)scene's cell and clock.
+// The new diagonal gradient of the stress servo (PeriTriaxController) from this step's
+// contacts: sums of their stress and stiffness in the cell Hp they were computed in.
+__device__ inline void servo_rates(const CellState *__restrict__ cs, const double *acc, double V,
+                                   double dt, double rate[3]) {
+  for (int a = 0; a < 3; ++a) {
+    if (cs->stress_mask & (1 << a)) {
+      const double sa = acc[a] / V, Ka = acc[3 + a] / V;
+      const double want = (1 - cs->grow_damping) * (cs->goal[a] - sa);
+      if (Ka > 0) rate[a] = want / (Ka * (dt * cs->glob_update));
+      else rate[a] = want > 0 ? cs->max_rate[a] : (want < 0 ? -cs->max_rate[a] : 0.0);
+      rate[a] = fmin(fmax(rate[a], -cs->max_rate[a]), cs->max_rate[a]);
+    } else {
+      rate[a] = cs->goal[a];
+    }
+  }
+}
+
+// Advance of a periodic cell whose matrices are all diagonal and stay so (sheared: every
+// off-diagonal entry of the state is an exact zero, and the servo writes the diagonal
+// only): the products reduce to one term an axis with the same values.  The kernel's time
+// is the latency of one thread, so everything is loaded before anything is stored and the
+// off-diagonal zeros are left alone.
+__device__ void cell_advance_diag(CellState *__restrict__ cs, const double *servo) {
+  double Hp[3], H[3], Lp[3], L[3], Hr[3], Hri[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    Hp[k] = cs->H[4 * k];
+    H[k] = cs->Hnext[4 * k];
+    Lp[k] = L[k] = cs->L[4 * k];
+    Hr[k] = cs->Href[4 * k];
+    Hri[k] = cs->Hrefinv[4 * k];
+  }
+  const double dt = cs->dt, time = cs->time, verlet = cs->verlet, rmax = cs->rmax;
+  const long long iter = cs->iter;
+  if (servo) {
+    const double V = fabs(Hp[0] * (Hp[1] * Hp[2]));
+    servo_rates(cs, servo, V, dt, L);
+  }
+  double e2 = 0, E[3], Hn[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    Hn[k] = __dmul_rn(__dadd_rn(1.0, __dmul_rn(L[k], dt)), H[k]);
+    E[k] = __dmul_rn(Hn[k] - Hr[k], Hri[k]);
+  }
+  for (int k = 0; k < 3; ++k) e2 += E[k] * E[k];
+  const double eff = verlet - sqrt(e2) * (rmax + verlet);
+  bool still = true;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int q = 4 * k;
+    const double W = __dmul_rn(Lp[k], Hp[k]), dL = L[k] - Lp[k];
+    still &= !nonzero_bits(dL);
+    cs->Hprev[q] = Hp[k];
+    cs->H[q] = H[k];
+    cs->Lprev[q] = Lp[k];
+    cs->L[q] = L[k];
+    cs->dL[q] = dL;
+    cs->W[q] = W;
+    cs->Hnext[q] = Hn[k];
+    cs->E[q] = E[k];
+    cs->Ef[q] = (float)E[k];
+    cs->Ep1[k] = 1.0 + E[k];
+    cs->dtL[k] = dt * L[k];
+    cs->dHf[q] = (float)(H[k] - Hr[k]);
+    cs->Wf[q] = (float)W;
+  }
+  cs->thr2 = eff > 0 ? eff * eff : -1.0;
+  cs->dl_zero = still;
+  cs->iter = iter + 1;
+  cs->time = __dadd_rn(time, dt);
+  cs->dt_law = dt;
+}
+
+// Advance of one (sub-)scene's cell and clock.  servo: the six sums of the stress servo on
+// its update steps (else null).
 __device__ void cell_advance(CellState *__restrict__ cs, const double *servo, P3d *p3d = nullptr) {
+  const bool steered = p3d && p3d->has_next;   // the Peri3dController's gradient takes over
+  if (cs->periodic && !cs->sheared && !steered) {
+    cell_advance_diag(cs, servo);
+    return;
+  }
   const double dt = cs->dt;
   if (cs->periodic) {
     double Hp[9], H[9], Lp[9], L[9], dL[9], W[9];
@@ -780,33 +961,17 @@ __device__ void cell_advance(CellState *__restrict__ cs, const double *servo, P3
       L[q] = Lp[q];
       dL[q] = 0.0;   // L - Lprev after the assignment above
     }
-    if (servo) {
-      // PeriTriaxController: new diagonal gradient from this step's contacts (their
-      // stress and stiffness in the cell Hprev they were computed in), effective from
-      // the next step; the partials are summed in block order
-      double acc[6] = {0, 0, 0, 0, 0, 0};
-      for (int b = 0; b < kServoBlocks; ++b)
-        for (int q = 0; q < 6; ++q) acc[q] += servo[6 * b + q];
+    if (servo) {   // effective from the next step
       const double V = fabs(Hp[0] * (Hp[4] * Hp[8] - Hp[5] * Hp[7]) -
                             Hp[1] * (Hp[3] * Hp[8] - Hp[5] * Hp[6]) +
                             Hp[2] * (Hp[3] * Hp[7] - Hp[4] * Hp[6]));
-      for (int a = 0; a < 3; ++a) {
-        double rate;
-        if (cs->stress_mask & (1 << a)) {
-          const double sa = acc[a] / V, Ka = acc[3 + a] / V;
-          const double want = (1 - cs->grow_damping) * (cs->goal[a] - sa);
-          if (Ka > 0) rate = want / (Ka * (dt * cs->glob_update));
-          else rate = want > 0 ? cs->max_rate[a] : (want < 0 ? -cs->max_rate[a] : 0.0);
-          rate = fmin(fmax(rate, -cs->max_rate[a]), cs->max_rate[a]);
-        } else {
-          rate = cs->goal[a];
-        }
-        L[4 * a] = rate;
-      }
+      double rate[3];
+      servo_rates(cs, servo, V, dt, rate);
+      for (int a = 0; a < 3; ++a) L[4 * a] = rate[a];
 #pragma unroll
       for (int q = 0; q < 9; ++q) dL[q] = L[q] - Lp[q];
     }
-    if (p3d && p3d->has_next) {
+    if (steered) {
       // the controller's gradient (k_p3d_update), effective from the next step like
       // Cell.velGrad
       for (int q = 0; q < 9; ++q) {
@@ -877,14 +1042,38 @@ __global__ void k_p3d_update(const CellState *cs, const DevStatus *ds, P3d *p3d,
 // One thread per sub-scene.  Every block reads "pending" before it counts itself
 // in; the last block to arrive (so every block has read it) turns a collider
 // request into "pending" and counts the step, so no block can see the flag of the
-// step it is advancing.
+// step it is advancing.  A single block needs no count.  The servo's partials (one block
+// of a scene without sub-scenes) are staged by the whole block and summed in block order
+// by a lane for each of the six sums: one thread loading and adding the 1824 of them took
+// about 50 us.
 __global__ void k_cell_advance(CellState *cs, int nsub, DevStatus *ds, const double *servo,
                                P3d *p3d) {
+  __shared__ double part[kServoBlocks * 6];
+  __shared__ double sums[6];
   const bool skip = *(volatile int *)&ds->pending;
+  const int request = *(volatile int *)&ds->request;   // set by the integrator, which is done
+  if (servo && !skip) {
+    for (int k = threadIdx.x; k < kServoBlocks * 6; k += blockDim.x) part[k] = servo[k];
+    __syncthreads();
+    if (threadIdx.x < 6) {
+      double acc = 0;
+#pragma unroll 8
+      for (int b = 0; b < kServoBlocks; ++b) acc += part[6 * b + threadIdx.x];
+      sums[threadIdx.x] = acc;
+    }
+    __syncthreads();
+  }
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (!skip && q < nsub && cs[q].alive)
-    cell_advance(cs + q, q == 0 ? servo : nullptr, q == 0 ? p3d : nullptr);
-  __syncthreads();
+    cell_advance(cs + q, servo && q == 0 ? sums : nullptr, q == 0 ? p3d : nullptr);
+  __syncthreads();   // every thread of the block has read "pending"
+  if (gridDim.x == 1) {
+    if (threadIdx.x == 0 && !skip) {
+      ds->steps += 1;
+      if (request) ds->pending = 1;
+    }
+    return;
+  }
   if (threadIdx.x == 0) {
     __threadfence();
     const int arrived = atomicAdd(&ds->arrive, 1);
@@ -892,7 +1081,7 @@ __global__ void k_cell_advance(CellState *cs, int nsub, DevStatus *ds, const dou
       ds->arrive = 0;
       if (!skip) {
         ds->steps += 1;
-        if (*(volatile int *)&ds->request) ds->pending = 1;
+        if (request) ds->pending = 1;
       }
     }
   }
@@ -1154,28 +1343,29 @@ void launch_dscale_reset(const Bodies &b, long long N, int multi, int sub, cudaS
 }
 
 void launch_integrate(const StepDesc *d, const StepDesc &h, bool desc, const CellState *cs,
-                      DevStatus *ds, const Mat *mats, int mixed, int block, cudaStream_t st) {
+                      DevStatus *ds, const Mat *mats, int mixed, int block, int nsm,
+                      cudaStream_t st) {
   const long long N = h.sc.N;
   if (N <= 0) return;
   const int feat = (h.sc.walls ? 1 : 0) | (h.sc.sheared ? 2 : 0);
+  block = spread_block(N, block, nsm);
+  const unsigned grid = (unsigned)((N + block - 1) / block);
   // kernels without the sphere-wall or sheared-cell branches when no sub-scene needs them
-#define DEM_I(K, B, F, D) K<B, F, D><<<(unsigned)((N + B - 1) / B), B, 0, st>>>(d, h, cs, ds, mats)
-#define DEM_I_F(K, B, D) switch (feat) { case 0: DEM_I(K, B, 0, D); break; case 1: DEM_I(K, B, 1, D); break; \
-                                         case 2: DEM_I(K, B, 2, D); break; default: DEM_I(K, B, 3, D); }
-#define DEM_I_B(K, D) if (block == 128) { DEM_I_F(K, 128, D) } else if (block == 512) { DEM_I_F(K, 512, D) } else { DEM_I_F(K, 256, D) }
+#define DEM_I(K, F, D) K<F, D><<<grid, block, 0, st>>>(d, h, cs, ds, mats)
+#define DEM_I_F(K, D) switch (feat) { case 0: DEM_I(K, 0, D); break; case 1: DEM_I(K, 1, D); break; \
+                                      case 2: DEM_I(K, 2, D); break; default: DEM_I(K, 3, D); }
   if (mixed) {
-    if (desc) { DEM_I_B(k_integrate_mixed, true) } else { DEM_I_B(k_integrate_mixed, false) }
+    if (desc) { DEM_I_F(k_integrate_mixed, true) } else { DEM_I_F(k_integrate_mixed, false) }
   } else {
-    if (desc) { DEM_I_B(k_integrate, true) } else { DEM_I_B(k_integrate, false) }
+    if (desc) { DEM_I_F(k_integrate, true) } else { DEM_I_F(k_integrate, false) }
   }
-#undef DEM_I_B
 #undef DEM_I_F
 #undef DEM_I
 }
 
 void launch_cell_advance(CellState *cs, int nsub, DevStatus *ds, const double *servo_partials,
                          cudaStream_t st, P3d *p3d, const double *p3d_partials) {
-  const int threads = nsub < 128 ? 32 * ((nsub + 31) / 32) : 128;
+  const int threads = servo_partials ? 256 : (nsub < 128 ? 32 * ((nsub + 31) / 32) : 128);
   if (p3d) k_p3d_update<<<1, 1, 0, st>>>(cs, ds, p3d, p3d_partials);
   k_cell_advance<<<(nsub + threads - 1) / threads, threads, 0, st>>>(cs, nsub, ds, servo_partials,
                                                                      p3d);

@@ -348,7 +348,7 @@ void drop_graphs(dem_scene *s) {
 void free_bodies(dem_scene *s, Bodies &b) {
   dfree(s, b.pos); dfree(s, b.vel); dfree(s, b.angvel); dfree(s, b.ori); dfree(s, b.xref);
   dfree(s, b.mprop); dfree(s, b.id); dfree(s, b.sid); dfree(s, b.mat); dfree(s, b.flags);
-  dfree(s, b.whist); dfree(s, b.rdsc);
+  dfree(s, b.whist); dfree(s, b.rdsc); dfree(s, b.live); dfree(s, b.wnear);
   dfree(s, b.p32); dfree(s, b.vw32); dfree(s, b.xref32); dfree(s, b.mprop32); dfree(s, b.ori32);
 }
 
@@ -359,7 +359,8 @@ dem_status alloc_bodies(dem_scene *s, Bodies &b, long long cap) {
       (r = dalloc(s, &b.xref, cap)) || (r = dalloc(s, &b.mprop, cap)) ||
       (r = dalloc(s, &b.id, cap)) || (r = dalloc(s, &b.sid, cap)) ||
       (r = dalloc(s, &b.mat, cap)) || (r = dalloc(s, &b.flags, cap)) ||
-      (r = dalloc(s, &b.rdsc, cap)))
+      (r = dalloc(s, &b.rdsc, cap)) || (r = dalloc(s, &b.live, cap)) ||
+      (r = dalloc(s, &b.wnear, cap)))
     return r;
   // wall histories exist for every body (a sub-scene with walls may join later)
   if ((r = dalloc(s, &b.whist, 6 * cap))) return r;
@@ -372,7 +373,7 @@ dem_status alloc_bodies(dem_scene *s, Bodies &b, long long cap) {
 
 void free_rows(dem_scene *s, Table &t) {
   dfree(s, t.pair); dfree(s, t.cpack); dfree(s, t.hfs); dfree(s, t.hn); dfree(s, t.oFM);
-  dfree(s, t.tanphi); dfree(s, t.down); dfree(s, t.found);
+  dfree(s, t.tanphi); dfree(s, t.down); dfree(s, t.found); dfree(s, t.bits);
   dfree(s, t.g32); dfree(s, t.hn32); dfree(s, t.oFM32); dfree(s, t.s0);
 }
 
@@ -391,7 +392,7 @@ dem_status ensure_table(dem_scene *s, Table &t, long long rows, long long nbody)
     free_rows(s, t);
     if ((r = dalloc(s, &t.pair, nc)) || (r = dalloc(s, &t.cpack, nc)) ||
         (r = dalloc(s, &t.hfs, nc)) || (r = dalloc(s, &t.down, nc)) ||
-        (r = dalloc(s, &t.found, nc)))
+        (r = dalloc(s, &t.found, nc)) || (r = dalloc(s, &t.bits, nc / 32 + 2)))
       return r;
     if (s->mixed) {
       if ((r = dalloc(s, &t.g32, nc)) || (r = dalloc(s, &t.hn32, nc)) || (r = dalloc(s, &t.s0, nc)) ||
@@ -783,7 +784,7 @@ dem_status rebuild_core(dem_scene *s) {
   exclusive_scan(s->cell_count, s->cell_start, ncell, s->scan_ws, s->st);
   launch_scatter(N, s->key, rank, s->cell_start, tmp, s->st);
   launch_reorder(s->cur, s->alt, n_live, s->cap, tmp, s->key, s->cell_start, raw, cr, s->new_to_old,
-                 s->slot_of_id, s->has_walls, s->mixed, id_shift, s->st);
+                 s->slot_of_id, s->has_walls, s->mixed, id_shift, s->cs_d, multi, s->st);
   std::swap(s->cur, s->alt);
   s->N = n_live;
   const long long NL = n_live;
@@ -896,7 +897,7 @@ long long scene_table_rows(const dem_scene *s) { return s ? s->tab[s->tc].P : 0;
 // ensure_table adds.
 double scene_bytes_per_body(int mixed) {
   const double d4 = sizeof(double4_32a), f4 = sizeof(float4);
-  double buf = 6 * d4 + 3 * sizeof(int) + sizeof(uint8_t) + sizeof(double) + 6 * d4;
+  double buf = 6 * d4 + 3 * sizeof(int) + 3 * sizeof(uint8_t) + sizeof(double) + 6 * d4;
   if (mixed) buf += 6 * f4;
   const double scratch = 5 * sizeof(int) + 2 * d4 + f4 + sizeof(int4) +
                         kCandKeep * sizeof(unsigned);
@@ -904,7 +905,7 @@ double scene_bytes_per_body(int mixed) {
   return 2 * buf + scratch + tables;
 }
 double scene_bytes_per_row(int mixed) {
-  double row = sizeof(int2) + sizeof(int) + sizeof(double4_32a) + 2 * sizeof(int);
+  double row = sizeof(int2) + sizeof(int) + sizeof(double4_32a) + 2 * sizeof(int) + 0.125;
   if (mixed) row += 2 * sizeof(float4) + 2 * sizeof(float4) + sizeof(float);
   else row += sizeof(double4_32a) + 2 * sizeof(double4_32a) + sizeof(double);
   return 2 * 1.25 * row;
@@ -1019,6 +1020,10 @@ dem_status dem_scene_create(const dem_scene_desc *desc, dem_scene **out) {
     dem_scene_destroy(s);
     return DEM_ERR_OOM;
   }
+  // The mixed integrator is bound by its loads: in slot order a warp's records are
+  // consecutive (1M dense spheres 112 us against 147 in degree order).  The FP64 one is
+  // bound by the FP64 pipe, which even row counts fill better (313 against 329 us).
+  s->degree_order = s->mixed ? 0 : 1;
   // sub-scene 0: the scene of the descriptor
   s->subs.resize(1);
   Sub &u0 = s->subs[0];
@@ -1402,7 +1407,7 @@ dem_status dem_step(dem_scene *s, long long nsteps) {
         }
         if (record) CK(cudaEventRecord(ev[6 * i + 2], s->st));
         launch_integrate(s->step_d, *s->step_h, desc, s->cs_d, s->ds_d, s->mats_d, s->mixed,
-                         s->integrate_block, s->st);
+                         s->integrate_block, s->nsm, s->st);
         if (record) { CK(cudaEventRecord(ev[6 * i + 3], s->st)); CK(cudaEventRecord(ev[6 * i + 4], s->st)); }
         // servo update steps (PeriTriaxController every glob_update steps)
         const bool upd = servo && ((it0 + i + 1) % s->cs0().glob_update == 0);
@@ -1984,7 +1989,7 @@ Bodies body_view(const Bodies &b, long long o) {
   Bodies v = b;
   auto sh = [o](auto *&p, long long k = 1) { if (p) p += k * o; };
   sh(v.pos); sh(v.vel); sh(v.angvel); sh(v.ori); sh(v.xref); sh(v.mprop);
-  sh(v.id); sh(v.sid); sh(v.mat); sh(v.flags); sh(v.whist); sh(v.rdsc);
+  sh(v.id); sh(v.sid); sh(v.mat); sh(v.flags); sh(v.live); sh(v.wnear); sh(v.whist); sh(v.rdsc);
   sh(v.p32); sh(v.vw32, 2); sh(v.xref32); sh(v.mprop32); sh(v.ori32);
   return v;
 }

@@ -81,3 +81,26 @@ def test_collider_run_carries_every_history(env, mixed):
         assert np.array_equal(ca["fs"], cb["fs"]) and np.array_equal(ca["fn"], cb["fn"])
     for s in (a, b):
         s.close()
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+def test_integrated_force_is_the_sum_over_all_rows(env, mixed):
+    """Undamped, without gravity, a step changes a velocity by dt F / m: the integrator's sum
+    over a body's real rows (masks of 32 rows; some bodies have more) against the query's sum
+    over all of them."""
+    torch, pkg = env
+    w = _cloud(3000, True)
+    w.damping = 0.0
+    s = _scene(pkg, w, precision=pkg.DEM_MIXED if mixed else pkg.DEM_FP64,
+               verlet_dist=0.5 * w.radius.min())
+    for _ in range(3):
+        v0 = s.state(force=False)["vel"]
+        s.step(1)
+        st = s.state()
+        m = w.materials[0].density * 4 / 3 * np.pi * w.radius ** 3
+        dv = 1e-9 * st["force"] / m[:, None]
+        # the velocity's own rounding, and in mixed precision the FP32 rounding of dt F / m
+        bound = 4e-16 * np.abs(st["vel"]) + (1e-6 if mixed else 1e-14) * np.abs(dv).max()
+        assert np.abs(dv).max() > 1e-6
+        assert np.all(np.abs(st["vel"] - v0 - dv) <= bound)
+    s.close()
