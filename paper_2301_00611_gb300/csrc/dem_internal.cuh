@@ -351,12 +351,12 @@ void launch_cell_advance(CellState *cs, int nsub, DevStatus *ds, const double *s
 // sum F_a (-l n_b)
 void launch_p3d_partials(const Table &t, const DevStatus *ds, int mixed, double *partials,
                          cudaStream_t st);
-// GlobalStiffnessTimeStepper: per-sub-scene minimum critical step (keys: nsub entries
-// preset to +inf bits, reset by the launch) applied to the due sub-scenes' dt
-void launch_timestepper(const Bodies &b, const Table &t, CellState *cs, int nsub,
-                        const DevStatus *ds, const Mat *mats, long long N, long long cap,
-                        int mixed, int multi, int walls, unsigned long long *keys,
-                        cudaStream_t st);
+// GlobalStiffnessTimeStepper (N > 0): per-sub-scene minimum critical step applied to the due
+// sub-scenes' dt.  keys, est_min: nsub entries preset to +inf (double, float bits), reset by
+// the launch; est: N floats of scratch, null to compute every body in FP64
+void launch_timestepper(const Bodies &b, const Table &t, CellState *cs, int nsub, DevStatus *ds,
+                        const Mat *mats, long long N, long long cap, int mixed, int multi, int walls,
+                        unsigned long long *keys, unsigned *est_min, float *est, cudaStream_t st);
 // servo: per-block sums of sigma_ii * V and K_i * V over the real rows (6 per block)
 void launch_servo_partials(const Table &t, const Bodies &b, const DevStatus *ds, int mixed, int law,
                            double *partials, cudaStream_t st);

@@ -194,6 +194,7 @@ struct dem_scene {
 
   Mat mats_h[kMaxMat]{};
   bool mat_set[kMaxMat]{};
+  double max_poisson = 0;        // of every material ever set
   Mat *mats_d = nullptr;
 
   long long N = 0, cap = 0;
@@ -242,7 +243,7 @@ struct dem_scene {
   Grid *grids_h = nullptr;       // pinned [subs_cap]
   int *shift_h = nullptr;        // pinned [subs_cap]
   unsigned long long *bbox_keys = nullptr;   // [6 * subs_cap]
-  unsigned long long *dt_keys = nullptr;     // [subs_cap] time-stepper minima (+inf bits)
+  unsigned long long *dt_keys = nullptr;     // [2 subs_cap] time-stepper minima, estimates
   unsigned long long *bbox_h = nullptr;      // pinned [6 * subs_cap]
   int subs_cap = 0;
   unsigned long long steps_seen = 0;   // DevStatus::steps at the last read
@@ -430,11 +431,13 @@ dem_status ensure_subs(dem_scene *s, int need) {
   s->cs_d = cs;
   dfree(s, s->grids_d); dfree(s, s->id_shift_d); dfree(s, s->bbox_keys); dfree(s, s->dt_keys);
   if ((r = dalloc(s, &s->grids_d, nc)) || (r = dalloc(s, &s->id_shift_d, nc)) ||
-      (r = dalloc(s, &s->bbox_keys, 6LL * nc)) || (r = dalloc(s, &s->dt_keys, nc)))
+      (r = dalloc(s, &s->bbox_keys, 6LL * nc)) || (r = dalloc(s, &s->dt_keys, 2LL * nc)))
     return r;
   {
-    std::vector<unsigned long long> inf(nc, 0x7ff0000000000000ull);
-    CK(cudaMemcpyAsync(s->dt_keys, inf.data(), sizeof(unsigned long long) * nc,
+    // +inf of doubles, then (in the second half) of floats
+    std::vector<unsigned long long> inf(2 * nc, 0x7ff0000000000000ull);
+    for (int q = nc; q < 2 * nc; ++q) inf[q] = 0x7f8000007f800000ull;
+    CK(cudaMemcpyAsync(s->dt_keys, inf.data(), sizeof(unsigned long long) * 2 * nc,
                        cudaMemcpyHostToDevice, s->st));
     if ((r = wait(s))) return r;
   }
@@ -1099,6 +1102,7 @@ dem_status dem_set_material(dem_scene *s, int mat, double density, double young,
   mindlin_compliances(m);
   s->mats_h[mat] = m;
   s->mat_set[mat] = true;
+  s->max_poisson = std::max(s->max_poisson, poisson);
   CK(cudaMemcpyAsync(s->mats_d + mat, &s->mats_h[mat], sizeof(Mat), cudaMemcpyHostToDevice, s->st));
   return sync_host(s);
 }
@@ -1384,6 +1388,8 @@ dem_status dem_step(dem_scene *s, long long nsteps) {
         if (u.used && u.cs.tstep && (u.cs.iter + i) % u.cs.tstep_interval == 0) return true;
       return false;
     };
+    // the stepper's FP32 estimates (in the force buffer, which queries use) need ks <= kn
+    float *est = s->max_poisson <= 1.0 ? reinterpret_cast<float *>(s->gT) : nullptr;
     // captured batches read the descriptor; launched ones take the arrays as parameters
     const bool use_graph = (s->step_graphs > 0 || (s->step_graphs < 0 && sc.N < kGraphAutoBodies)) &&
                            !ev && !servo && !tstep && !p3d;
@@ -1402,8 +1408,9 @@ dem_status dem_step(dem_scene *s, long long nsteps) {
         if (record) CK(cudaEventRecord(ev[6 * i + 1], s->st));
         if (tstep && tstep_due(i)) {   // GlobalStiffnessTimeStepper: after the contacts
           launch_timestepper(s->cur, t, s->cs_d, s->nsub(), s->ds_d, s->mats_d, sc.N, s->cap,
-                             s->mixed, sc.multi, sc.walls, s->dt_keys, s->st);
-          s->launches += 2;
+                             s->mixed, sc.multi, sc.walls, s->dt_keys,
+                             reinterpret_cast<unsigned *>(s->dt_keys + s->subs_cap), est, s->st);
+          s->launches += est ? 2 : 1;
         }
         if (record) CK(cudaEventRecord(ev[6 * i + 2], s->st));
         launch_integrate(s->step_d, *s->step_h, desc, s->cs_d, s->ds_d, s->mats_d, s->mixed,
