@@ -363,13 +363,30 @@ void launch_servo_partials(const Table &t, const Bodies &b, const DevStatus *ds,
 void launch_gather_forces(const Bodies &b, const Table &t, const Mat *mats, const CellState *cs,
                           const SceneConst &sc, long long cap, double4_32a *F, double4_32a *T,
                           int mixed, cudaStream_t st);
-// dst[i] = src[slot_of_id[i]] for i < n (records of consecutive ids, in id order)
 // density scaling switched off: factor 1 for the bodies of sub-scene `sub` (all unless multi)
 void launch_dscale_reset(const Bodies &b, long long N, int multi, int sub, cudaStream_t st);
-void launch_gather_ids(const int *slot_of_id, long long n, const double4_32a *src,
-                       double4_32a *dst, cudaStream_t st);
-void launch_gather_ids_f(const int *slot_of_id, long long n, const float4 *src, float4 *dst,
-                         cudaStream_t st);
+// export.cu: bodies in id order (null destinations are left out; orientations from ori32
+// when set), and contacts in (id1, id2) order
+struct StatePack {
+  const double4_32a *src3[3];   // position, velocity, spin records by slot
+  double *dst3[3];              // three doubles an id
+  const double4_32a *ori64;
+  const float4 *ori32;
+  double4_32a *ori;
+};
+void launch_state_pack(const int *slot_of_id, long long n, const StatePack &a, cudaStream_t st);
+struct ContactPack {
+  int *id1, *id2, *c;
+  double *fn, *fs, *n, *cp, *phys, *pen;
+};
+// cnt: N counts, or 7 N with walls (walls 5..0 first)
+void launch_contact_count(const int *slot_of_id, const Bodies &b, const Table &t, long long N,
+                          int mixed, int walls, int *cnt, cudaStream_t st);
+// off: the exclusive prefix sum of cnt with its total; contacts [first, first + count)
+void launch_contact_emit(const int *slot_of_id, const Bodies &b, const Table &t, long long N,
+                         long long cap, int mixed, int walls, int multi, const CellState *cs,
+                         const Mat *mats, const int *off, long long first, long long count,
+                         const ContactPack &o, cudaStream_t st);
 // micro.cu: fabric / normal-shear stress partials (28 per block, micro_blocks(P) blocks)
 // and per-body stress tensors (9 per slot)
 int micro_blocks(long long P);

@@ -1511,26 +1511,6 @@ void launch_gather_forces(const Bodies &b, const Table &t, const Mat *mats, cons
     k_gather_forces<<<blocks(sc.N), kT, 0, st>>>(b, t, mats, cs, sc, cap, F, T, mixed);
 }
 
-__global__ void k_gather_ids(const int *__restrict__ slot_of_id, long long n,
-                             const double4_32a *__restrict__ src, double4_32a *dst) {
-  const long long i = (long long)blockIdx.x * kT + threadIdx.x;
-  if (i < n) dst[i] = src[slot_of_id[i]];
-}
-__global__ void k_gather_ids_f(const int *__restrict__ slot_of_id, long long n,
-                               const float4 *__restrict__ src, float4 *dst) {
-  const long long i = (long long)blockIdx.x * kT + threadIdx.x;
-  if (i < n) dst[i] = src[slot_of_id[i]];
-}
-
-void launch_gather_ids(const int *slot_of_id, long long n, const double4_32a *src,
-                       double4_32a *dst, cudaStream_t st) {
-  if (n > 0) k_gather_ids<<<blocks(n), kT, 0, st>>>(slot_of_id, n, src, dst);
-}
-void launch_gather_ids_f(const int *slot_of_id, long long n, const float4 *src, float4 *dst,
-                         cudaStream_t st) {
-  if (n > 0) k_gather_ids_f<<<blocks(n), kT, 0, st>>>(slot_of_id, n, src, dst);
-}
-
 int stats_blocks(long long n) {
   long long b = (n + kT - 1) / kT;
   return (int)(b < 1 ? 1 : (b > 1024 ? 1024 : b));

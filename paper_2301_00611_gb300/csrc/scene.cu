@@ -21,6 +21,9 @@
 #include <unordered_map>
 #include <vector>
 
+#include <sys/mman.h>
+#include <unistd.h>
+
 #include "dem_internal.cuh"
 #include "dem.h"
 
@@ -1506,19 +1509,80 @@ dem_status dem_step(dem_scene *s, long long nsteps) {
   return DEM_OK;
 }
 
-static dem_status fetch4(dem_scene *s, const double4_32a *src, const std::vector<int> &sid, double *out,
-                         int comps) {
-  const long long N = s->N;
-  std::vector<double4_32a> h(N);
-  CK(cudaMemcpyAsync(h.data(), src, sizeof(double4_32a) * N, cudaMemcpyDeviceToHost, s->st));
-  dem_status r = wait(s);
-  if (r) return r;
-  for (long long i = 0; i < N; ++i) {
-    const double4_32a &v = h[sid[i]];
-    const double c[4] = {v.x, v.y, v.z, v.w};
-    for (int k = 0; k < comps; ++k) out[comps * i + k] = c[k];
+// The copies to a caller's arrays go straight to its pages.  Pages that were never touched
+// (a freshly allocated array) fault one by one under the copy, which took 21 to 37 ms for the
+// state of a million spheres against 0.7 ms into touched pages; the processor maps them
+// several times faster.  A few pages are sampled; where one is missing, every page of the
+// range is touched (its contents are about to be overwritten), by a few threads when large.
+static void touch_fresh(void *dst, size_t bytes) {
+  static const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+  if (!dst || bytes < 16 * page) return;
+  char *const p = static_cast<char *>(dst);
+  const size_t lead = reinterpret_cast<uintptr_t>(p) % page, pages = (lead + bytes + page - 1) / page;
+  bool fresh = false;
+  for (size_t k = 0; k < 16 && !fresh; ++k) {
+    unsigned char in = 1;
+    fresh = mincore(p - lead + page * (k * (pages - 1) / 15), 1, &in) == 0 && !(in & 1);
   }
-  return DEM_OK;
+  if (!fresh) return;
+  auto touch = [=](size_t a, size_t b) {
+    for (size_t k = a; k < b; ++k) *const_cast<volatile char *>(k ? p - lead + page * k : p) = 0;
+  };
+  const size_t parts = std::min<size_t>(8, 1 + bytes / (4u << 20));
+  std::vector<std::thread> helpers;
+  size_t done = 0;   // pages [0, done) are taken by helpers
+  try {
+    helpers.reserve(parts);
+    for (size_t k = 0; k + 1 < parts; ++k) {
+      const size_t to = pages * (k + 1) / parts;
+      helpers.emplace_back(touch, done, to);
+      done = to;
+    }
+  } catch (...) {   // no more threads: the rest here
+  }
+  touch(done, pages);
+  for (auto &h : helpers) h.join();
+}
+
+// Bodies [first, first + n) in id order to the caller's arrays: packed on the device into
+// the collider's list buffer (scratch between its runs; 104 of its 128 bytes a body), then
+// one copy an array.
+constexpr size_t kStagingBytes = 1024 * 32 * sizeof(double);   // of partials_h
+static_assert(kCandKeep * sizeof(unsigned) >= 9 * sizeof(double) + sizeof(double4_32a),
+              "the list buffer holds a packed state");
+static dem_status export_state(dem_scene *s, long long first, long long n, const double4_32a *pos_d,
+                               const double4_32a *vel_d, const double4_32a *ang_d, double *pos,
+                               double *vel, double *angvel, double *ori) {
+  char *buf = reinterpret_cast<char *>(s->cand_list);
+  double4_32a *o = reinterpret_cast<double4_32a *>(buf);
+  double *d[3];
+  for (int k = 0; k < 3; ++k) d[k] = reinterpret_cast<double *>(buf + 32 * n) + 3 * n * k;
+  StatePack a{{pos_d, vel_d, ang_d},
+              {pos ? d[0] : nullptr, vel ? d[1] : nullptr, angvel ? d[2] : nullptr},
+              s->cur.ori, s->mixed ? s->cur.ori32 : nullptr, ori ? o : nullptr};
+  launch_state_pack(s->slot_of_id + first, n, a, s->st);
+  CK(cudaGetLastError());
+  double *out[3] = {pos, vel, angvel};
+  const size_t bytes = (sizeof(double4_32a) + 9 * sizeof(double)) * n;
+  if (bytes <= kStagingBytes) {
+    // a copy into pageable memory takes some 14 us however small: one copy through pinned
+    // memory instead of four
+    char *h = reinterpret_cast<char *>(s->partials_h);
+    CK(cudaMemcpyAsync(h, buf, bytes, cudaMemcpyDeviceToHost, s->st));
+    const dem_status r = wait(s);
+    if (r) return r;
+    for (int k = 0; k < 3; ++k)
+      if (out[k]) std::memcpy(out[k], h + 32 * n + 24 * n * k, sizeof(double) * 3 * n);
+    if (ori) std::memcpy(ori, h, sizeof(double) * 4 * n);
+    return DEM_OK;
+  }
+  for (int k = 0; k < 3; ++k) touch_fresh(out[k], sizeof(double) * 3 * n);
+  touch_fresh(ori, sizeof(double) * 4 * n);
+  for (int k = 0; k < 3; ++k)
+    if (out[k])
+      CK(cudaMemcpyAsync(out[k], d[k], sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, s->st));
+  if (ori) CK(cudaMemcpyAsync(ori, o, sizeof(double) * 4 * n, cudaMemcpyDeviceToHost, s->st));
+  return wait(s);
 }
 
 static dem_status fetch_sid(dem_scene *s, std::vector<int> &sid) {
@@ -1534,24 +1598,9 @@ dem_status dem_get_state(dem_scene *s, double *pos, double *vel, double *angvel,
   dem_status r;
   if ((r = sync_host(s))) return r;
   if (s->N == 0) return DEM_OK;
-  std::vector<int> sid;
-  if ((r = fetch_sid(s, sid))) return r;
-  if (pos && (r = fetch4(s, s->cur.pos, sid, pos, 3))) return r;
-  if (vel && (r = fetch4(s, s->cur.vel, sid, vel, 3))) return r;
-  if (angvel && (r = fetch4(s, s->cur.angvel, sid, angvel, 3))) return r;
-  if (ori) {
-    if (s->mixed) {
-      std::vector<float4> h(s->N);
-      CK(cudaMemcpyAsync(h.data(), s->cur.ori32, sizeof(float4) * s->N, cudaMemcpyDeviceToHost, s->st));
-      if ((r = wait(s))) return r;
-      for (long long i = 0; i < s->N; ++i) {
-        const float4 &q = h[sid[i]];
-        ori[4 * i] = q.x; ori[4 * i + 1] = q.y; ori[4 * i + 2] = q.z; ori[4 * i + 3] = q.w;
-      }
-    } else if ((r = fetch4(s, s->cur.ori, sid, ori, 4))) {
-      return r;
-    }
-  }
+  if ((pos || vel || angvel || ori) &&
+      (r = export_state(s, 0, s->N, s->cur.pos, s->cur.vel, s->cur.angvel, pos, vel, angvel, ori)))
+    return r;
   if (force || torque) {
     if (!s->table_fresh) {
       // no contact table matches the current body order yet: no contact forces
@@ -1562,8 +1611,8 @@ dem_status dem_get_state(dem_scene *s, double *pos, double *vel, double *angvel,
     launch_gather_forces(s->cur, s->tab[s->tc], s->mats_d, s->cs_d, scene_const(s), s->cap,
                          s->gF, s->gT, s->mixed, s->st);
     CK(cudaGetLastError());
-    if (force && (r = fetch4(s, s->gF, sid, force, 3))) return r;
-    if (torque && (r = fetch4(s, s->gT, sid, torque, 3))) return r;
+    if ((r = export_state(s, 0, s->N, s->gF, s->gT, nullptr, force, torque, nullptr, nullptr)))
+      return r;
   }
   return DEM_OK;
 }
@@ -1677,157 +1726,36 @@ dem_status dem_set_clock(dem_scene *s, long long iter, double time) {
 }
 
 namespace {
-struct HostContact {
-  int id1, id2, c[3];
-  double fn[3], fs[3], n[3], cp[3], phys[3], pen;
-};
-
-void wall_phys_h(const dem_scene *s, int wmat, int mat, double r, double &kn, double &ks,
-                 double &tp, int law) {
-  const Mat &mw = s->mats_h[wmat], &ms = s->mats_h[mat];
-  tp = std::min(mw.tanphi, ms.tanphi);
-  if (law) {   // Hertz-Mindlin constants kno, kso with an infinite wall radius
-    mindlin_phys(ms, r, mw, -1.0, kn, ks);
-    return;
-  }
-  double k1 = mw.young * (2 * r), k2 = ms.young * (2 * r);
-  kn = k1 * k2 / (k1 + k2);
-  double s1 = mw.young * mw.poisson * (2 * r), s2 = ms.young * ms.poisson * (2 * r);
-  ks = s1 * s2 / (s1 + s2);
-}
-
-dem_status collect_contacts(dem_scene *s, std::vector<HostContact> &out) {
-  out.clear();
+// Contacts counted on the device: prefix sums of the counts (id by id; walls 5..0 first) in
+// the collider's list buffer, which is scratch between its runs.  *total: their number.
+dem_status count_contacts(dem_scene *s, const int **off, long long *total) {
+  *total = 0;
   dem_status r;
   if ((r = sync_host(s))) return r;
   const long long N = s->N;
   if (N == 0 || !s->table_fresh) return DEM_OK;
-  const Table &t = s->tab[s->tc];
-  const long long P = t.P;
-  std::vector<int2> pair(P);
-  std::vector<int> cp(P), id(N);
-  std::vector<double4_32a> hfs(P), hn(P), oF(P), oM(P), oFM, pos(N);
-  std::vector<double> tp(P);
-  std::vector<float4> g32, hn32, oFM32;
-  if (P > 0) {
-    CK(cudaMemcpyAsync(pair.data(), t.pair, sizeof(int2) * P, cudaMemcpyDeviceToHost, s->st));
-    CK(cudaMemcpyAsync(cp.data(), t.cpack, sizeof(int) * P, cudaMemcpyDeviceToHost, s->st));
-    CK(cudaMemcpyAsync(hfs.data(), t.hfs, sizeof(double4_32a) * P, cudaMemcpyDeviceToHost, s->st));
-    if (s->mixed) {
-      g32.resize(P); hn32.resize(P); oFM32.resize(2 * P);
-      CK(cudaMemcpyAsync(g32.data(), t.g32, sizeof(float4) * P, cudaMemcpyDeviceToHost, s->st));
-      CK(cudaMemcpyAsync(hn32.data(), t.hn32, sizeof(float4) * P, cudaMemcpyDeviceToHost, s->st));
-      CK(cudaMemcpyAsync(oFM32.data(), t.oFM32, sizeof(float4) * 2 * P, cudaMemcpyDeviceToHost, s->st));
-    } else {
-      CK(cudaMemcpyAsync(hn.data(), t.hn, sizeof(double4_32a) * P, cudaMemcpyDeviceToHost, s->st));
-      oFM.resize(2 * P);
-      CK(cudaMemcpyAsync(oFM.data(), t.oFM, sizeof(double4_32a) * 2 * P, cudaMemcpyDeviceToHost, s->st));
-      CK(cudaMemcpyAsync(tp.data(), t.tanphi, sizeof(double) * P, cudaMemcpyDeviceToHost, s->st));
-    }
-  }
-  CK(cudaMemcpyAsync(id.data(), s->cur.id, sizeof(int) * N, cudaMemcpyDeviceToHost, s->st));
-  CK(cudaMemcpyAsync(pos.data(), s->cur.pos, sizeof(double4_32a) * N, cudaMemcpyDeviceToHost, s->st));
-  std::vector<uint8_t> flags(N);
-  std::vector<double4_32a> wh;
-  CK(cudaMemcpyAsync(flags.data(), s->cur.flags, N, cudaMemcpyDeviceToHost, s->st));
-  if (s->has_walls) {
-    wh.resize(6 * N);
-    for (int w = 0; w < 6; ++w)
-      CK(cudaMemcpyAsync(wh.data() + w * N, s->cur.whist + w * s->cap, sizeof(double4_32a) * N,
-                         cudaMemcpyDeviceToHost, s->st));
-  }
+  // 32 ints a body, at least 1024 bodies: counts (7 N), their sums (7 N + 1), scan workspace
+  int *buf = reinterpret_cast<int *>(s->cand_list);
+  const long long runs = s->has_walls ? 7 * N : N;
+  int *cnt = buf, *sum = buf + 8 * s->cap, *ws = buf + 16 * s->cap;
+  launch_contact_count(s->slot_of_id, s->cur, s->tab[s->tc], N, s->mixed, s->has_walls, cnt, s->st);
+  exclusive_scan(cnt, sum, runs, ws, s->st);
+  CK(cudaGetLastError());
+  CK(cudaMemcpyAsync(&s->rb_h->totals[0], sum + runs, sizeof(int), cudaMemcpyDeviceToHost, s->st));
   if ((r = wait(s))) return r;
-  if (s->mixed) {   // one view of both layouts: hfs = (Fs, kn), hn = (n, ks), tp = tan(phi)
-    for (long long k = 0; k < P; ++k) {
-      tp[k] = hfs[k].w;
-      hfs[k].w = g32[k].w;
-      hn[k] = make_double4_32a(hn32[k].x, hn32[k].y, hn32[k].z, hn32[k].w);
-      const float4 f = oFM32[2 * k], m = oFM32[2 * k + 1];
-      oF[k] = make_double4_32a(f.x, f.y, f.z, f.w);
-      oM[k] = make_double4_32a(m.x, m.y, m.z, m.w);
-    }
-  } else {
-    for (long long k = 0; k < P; ++k) {
-      oF[k] = oFM[2 * k];
-      oM[k] = oFM[2 * k + 1];
-    }
-  }
-  for (long long k = 0; k < P; ++k) {
-    if (hfs[k].w == 0.0) continue;
-    HostContact h{};
-    int a = pair[k].x, b = pair[k].y;
-    int c0, c1, c2;
-    unpack_shift(cp[k], c0, c1, c2);
-    double sg = 1.0;
-    const double F[3] = {oF[k].x, oF[k].y, oF[k].z};
-    const double fs[3] = {hfs[k].x, hfs[k].y, hfs[k].z};
-    const double n[3] = {hn[k].x, hn[k].y, hn[k].z};
-    const double d1 = oF[k].w;
-    const double r1 = pos[a].w;
-    const double pen = 2.0 * (r1 - d1);
-    if (id[a] < id[b]) {
-      h.id1 = id[a]; h.id2 = id[b]; h.c[0] = c0; h.c[1] = c1; h.c[2] = c2;
-    } else {
-      h.id1 = id[b]; h.id2 = id[a]; h.c[0] = -c0; h.c[1] = -c1; h.c[2] = -c2; sg = -1.0;
-    }
-    for (int q = 0; q < 3; ++q) {
-      h.fs[q] = sg * fs[q];
-      h.fn[q] = sg * (F[q] - fs[q]);
-      h.n[q] = sg * n[q];
-    }
-    // contact point x1 + (r1 - pen/2) n from the current position of the slot-first body
-    const double pa[3] = {pos[a].x, pos[a].y, pos[a].z};
-    for (int q = 0; q < 3; ++q) h.cp[q] = pa[q] + d1 * n[q];
-    h.phys[0] = hfs[k].w; h.phys[1] = hn[k].w; h.phys[2] = tp[k];
-    h.pen = pen;
-    out.push_back(h);
-  }
-  if (s->has_walls) {
-    std::vector<int> wmat(N, 0), wlaw(N, 0);   // wall material and law of each id's sub-scene
-    for (const Sub &u : s->subs)
-      if (u.used || u.removing)
-        for (long long i = u.id0; i < u.id0 + u.n && i < N; ++i) {
-          wmat[i] = u.cs.wall_mat;
-          wlaw[i] = u.cs.law;
-        }
-    for (long long sl = 0; sl < N; ++sl) {
-      if (!(flags[sl] & 0x7e)) continue;
-      for (int w = 0; w < 6; ++w) {
-        if (!(flags[sl] & (2 << w))) continue;
-        const double4_32a hw = wh[w * N + sl];
-        HostContact h{};
-        int ax = w >> 1;
-        double sn = hw.w >= 0 ? 1.0 : -1.0, Fn = std::fabs(hw.w);
-        h.id1 = -(w + 1);
-        h.id2 = id[sl];
-        double kn, ks, tanp;
-        const double rr = pos[sl].w;
-        const int law = wlaw[id[sl]];
-        wall_phys_h(s, wmat[id[sl]], s->mat_h[id[sl]], rr, kn, ks, tanp, law);
-        h.n[ax] = sn;
-        h.fn[ax] = sn * Fn;
-        h.fs[0] = hw.x; h.fs[1] = hw.y; h.fs[2] = hw.z;
-        h.pen = wall_pen(Fn, kn, law);
-        const double pp[3] = {pos[sl].x, pos[sl].y, pos[sl].z};
-        for (int q = 0; q < 3; ++q) h.cp[q] = pp[q] - (rr - 0.5 * h.pen) * h.n[q];
-        h.phys[0] = kn; h.phys[1] = ks; h.phys[2] = tanp;
-        out.push_back(h);
-      }
-    }
-  }
-  std::sort(out.begin(), out.end(), [](const HostContact &x, const HostContact &y) {
-    return x.id1 != y.id1 ? x.id1 < y.id1 : x.id2 < y.id2;
-  });
+  *off = sum;
+  *total = s->rb_h->totals[0];
   return DEM_OK;
 }
 }  // namespace
 
 dem_status dem_count_contacts(dem_scene *s, long long *count) {
   if (!s || !count) return DEM_ERR_INVALID_ARG;
-  std::vector<HostContact> v;
-  dem_status r = collect_contacts(s, v);
+  const int *off = nullptr;
+  long long total = 0;
+  dem_status r = count_contacts(s, &off, &total);
   if (r) return r;
-  *count = (long long)v.size();
+  *count = total;
   return DEM_OK;
 }
 
@@ -1836,26 +1764,57 @@ dem_status dem_get_contacts(dem_scene *s, long long cap, long long *count, int *
                             double *normal, double *contact_point, double *phys, double *pen) {
   if (!s) return DEM_ERR_INVALID_ARG;
   if (cap < 0) return fail(s, DEM_ERR_INVALID_ARG, "negative capacity");
-  std::vector<HostContact> v;
-  dem_status r = collect_contacts(s, v);
+  const int *off = nullptr;
+  long long total = 0;
+  dem_status r = count_contacts(s, &off, &total);
   if (r) return r;
-  if (count) *count = (long long)v.size();
-  long long m = std::min<long long>(cap, (long long)v.size());
-  for (long long k = 0; k < m; ++k) {
-    const HostContact &h = v[k];
-    if (id1) id1[k] = h.id1;
-    if (id2) id2[k] = h.id2;
-    for (int q = 0; q < 3; ++q) {
-      if (cell_dist) cell_dist[3 * k + q] = h.c[q];
-      if (normal_force) normal_force[3 * k + q] = h.fn[q];
-      if (shear_force) shear_force[3 * k + q] = h.fs[q];
-      if (normal) normal[3 * k + q] = h.n[q];
-      if (contact_point) contact_point[3 * k + q] = h.cp[q];
-      if (phys) phys[3 * k + q] = h.phys[q];
-    }
-    if (pen) pen[k] = h.pen;
+  if (count) *count = total;
+  const long long m = std::min<long long>(cap, total);
+  // records go through a device buffer a chunk at a time (148 bytes a contact), smaller
+  // where the memory left does not hold the usual chunk
+  long long chunk = std::min<long long>(m, 1LL << 20);
+  char *buf = nullptr;
+  const long long rec = 3 * 8 * 5 + 8 + 4 + 4 + 12;
+  while (m > 0 && !buf) {
+    r = dalloc(s, &buf, chunk * rec);
+    if (r && chunk <= 1024) return r;
+    if (r) chunk = std::max<long long>(chunk / 8, 1024);
   }
-  return DEM_OK;
+  for (long long at = 0; at < m && !r; at += chunk) {
+    const long long k = std::min(chunk, m - at);
+    double *d = reinterpret_cast<double *>(buf);
+    ContactPack o{};
+    o.fn = d; o.fs = d + 3 * k; o.n = d + 6 * k; o.cp = d + 9 * k; o.phys = d + 12 * k;
+    o.pen = d + 15 * k;
+    int *q = reinterpret_cast<int *>(d + 16 * k);
+    o.id1 = q; o.id2 = q + k; o.c = q + 2 * k;
+    launch_contact_emit(s->slot_of_id, s->cur, s->tab[s->tc], s->N, s->cap, s->mixed, s->has_walls,
+                        s->nsub() > 1, s->cs_d, s->mats_d, off, at, k, o, s->st);
+    struct Out { void *dst; const void *src; size_t each; };
+    const Out outs[] = {{id1, o.id1, 4}, {id2, o.id2, 4}, {cell_dist, o.c, 12},
+                        {normal_force, o.fn, 24}, {shear_force, o.fs, 24}, {normal, o.n, 24},
+                        {contact_point, o.cp, 24}, {phys, o.phys, 24}, {pen, o.pen, 8}};
+    cudaError_t e = cudaGetLastError();
+    if (rec * k <= (long long)kStagingBytes && e == cudaSuccess) {   // as export_state
+      char *h = reinterpret_cast<char *>(s->partials_h);
+      e = cudaMemcpyAsync(h, buf, rec * k, cudaMemcpyDeviceToHost, s->st);
+      r = e == cudaSuccess ? wait(s) : cuda_fail(s, e, "contact export");
+      for (const Out &x : outs)
+        if (x.dst && !r)
+          std::memcpy(static_cast<char *>(x.dst) + x.each * at,
+                      h + (static_cast<const char *>(x.src) - buf), x.each * k);
+      continue;
+    }
+    for (const Out &x : outs)
+      if (x.dst) touch_fresh(static_cast<char *>(x.dst) + x.each * at, x.each * k);
+    for (const Out &x : outs)
+      if (x.dst && e == cudaSuccess)
+        e = cudaMemcpyAsync(static_cast<char *>(x.dst) + x.each * at, x.src, x.each * k,
+                            cudaMemcpyDeviceToHost, s->st);
+    r = e == cudaSuccess ? wait(s) : cuda_fail(s, e, "contact export");
+  }
+  dfree(s, buf);
+  return r;
 }
 
 dem_status dem_set_contacts(dem_scene *s, long long n, const int *id1, const int *id2,
@@ -2424,38 +2383,7 @@ dem_status dem_get_state_range(dem_scene *s, long long first_id, long long n, do
   dem_status r;
   if ((r = sync_host(s))) return r;
   if (n == 0) return DEM_OK;
-  std::vector<double4_32a> h(n);
-  auto get = [&](const double4_32a *src, double *out, int comps) -> dem_status {
-    launch_gather_ids(s->slot_of_id + first_id, n, src, s->gT, s->st);
-    CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(h.data(), s->gT, sizeof(double4_32a) * n, cudaMemcpyDeviceToHost, s->st));
-    dem_status q = wait(s);
-    if (q) return q;
-    for (long long i = 0; i < n; ++i) {
-      const double c[4] = {h[i].x, h[i].y, h[i].z, h[i].w};
-      for (int k = 0; k < comps; ++k) out[comps * i + k] = c[k];
-    }
-    return DEM_OK;
-  };
-  if (pos && (r = get(s->cur.pos, pos, 3))) return r;
-  if (vel && (r = get(s->cur.vel, vel, 3))) return r;
-  if (angvel && (r = get(s->cur.angvel, angvel, 3))) return r;
-  if (ori) {
-    if (s->mixed) {
-      std::vector<float4> f(n);
-      launch_gather_ids_f(s->slot_of_id + first_id, n, s->cur.ori32, reinterpret_cast<float4 *>(s->gT),
-                          s->st);
-      CK(cudaGetLastError());
-      CK(cudaMemcpyAsync(f.data(), s->gT, sizeof(float4) * n, cudaMemcpyDeviceToHost, s->st));
-      if ((r = wait(s))) return r;
-      for (long long i = 0; i < n; ++i) {
-        ori[4 * i] = f[i].x; ori[4 * i + 1] = f[i].y; ori[4 * i + 2] = f[i].z; ori[4 * i + 3] = f[i].w;
-      }
-    } else if ((r = get(s->cur.ori, ori, 4))) {
-      return r;
-    }
-  }
-  return DEM_OK;
+  return export_state(s, first_id, n, s->cur.pos, s->cur.vel, s->cur.angvel, pos, vel, angvel, ori);
 }
 
 // ------------------------------------------------------------------ micromechanics
