@@ -396,11 +396,10 @@ void launch_body_stress(const Bodies &b, const Table &t, long long N, long long 
                         cudaStream_t st);
 // stats: per-block partial sums (deterministic tree), summed on the host in block order
 int stats_blocks(long long n);
-void launch_body_stats(const Bodies &b, const double4_32a *F, long long N, double *partials,
-                       cudaStream_t st);
-void launch_row_stats(const Table &t, const Bodies &b, double *partials, int mixed,
-                      cudaStream_t st);
-void launch_wall_stats(const Bodies &b, const SceneConst &sc, const Mat *mats, long long cap,
-                       double *partials, cudaStream_t st);
+// bodies [s0, s0 + n) on nbody blocks and, with a table, the rows they own on nrow blocks:
+// 5 nbody + 11 nrow partials, then (nrow > 0) the number of rows
+void launch_stats(const Bodies &b, const Table &t, const Mat *mats, const CellState *cs,
+                  const SceneConst &sc, long long cap, long long s0, long long n, int table,
+                  int mixed, int nbody, int nrow, double *partials, cudaStream_t st);
 
 }  // namespace dem

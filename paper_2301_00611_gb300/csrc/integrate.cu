@@ -1145,65 +1145,85 @@ __device__ inline void block_reduce_store(double (&v)[K], double *partials) {
     for (int q = 0; q < K; ++q) partials[K * blockIdx.x + q] = sh[q][0];
 }
 
-// ke, sum |F contact| over free bodies, number of free bodies
-__global__ void k_body_stats(Bodies b, const double4_32a *__restrict__ F, long long N, double *partials) {
-  double v[3] = {0, 0, 0};
-  for (long long i = (long long)blockIdx.x * kT + threadIdx.x; i < N; i += (long long)gridDim.x * kT) {
-    const double4_32a u = b.vel[i], w = b.angvel[i], mp = b.mprop[i];
-    v[0] += 0.5 * mp.x * (u.x * u.x + u.y * u.y + u.z * u.z) + 0.5 * mp.y * (w.x * w.x + w.y * w.y + w.z * w.z);
-    if (!(b.flags[i] & 1)) {
-      const double4_32a f = F[i];
-      v[1] += sqrt(f.x * f.x + f.y * f.y + f.z * f.z);
-      v[2] += 1.0;
+// Statistics of bodies [s0, s0 + n) and of the rows they own, in one launch: the first nbody
+// blocks take the bodies (kinetic energy, sum of |contact force| over free bodies, free
+// bodies, wall contacts, sum of their |F|), the others the real rows (count, sum |F|,
+// Love-Weber stress sum F_i (x1 - x2')_j).  Partials: 5 a body block, then 11 a row block,
+// then the number of rows.
+//
+// Separate passes (forces of every body to memory, body sums, row sums, wall sums, a copy and
+// a wait after each) cost a look at a small scene three round trips: 20k spheres 81 -> 49 us,
+// 1M dense 586 -> 396.
+__global__ void __launch_bounds__(kT) k_stats(Bodies b, Table t, const Mat *__restrict__ mats,
+                                              const CellState *__restrict__ cs, SceneConst sc,
+                                              long long cap, long long s0, long long n, int table,
+                                              int mixed, int nbody, double *partials) {
+  if ((int)blockIdx.x < nbody) {
+    double v[5] = {0, 0, 0, 0, 0};
+    for (long long i = (long long)blockIdx.x * kT + threadIdx.x; i < n; i += (long long)nbody * kT) {
+      const int s = (int)(s0 + i);
+      const double4_32a u = b.vel[s], w = b.angvel[s], mp = b.mprop[s];
+      v[0] += 0.5 * mp.x * (u.x * u.x + u.y * u.y + u.z * u.z) +
+              0.5 * mp.y * (w.x * w.x + w.y * w.y + w.z * w.z);
+      const uint8_t fl = b.flags[s];
+      double F[3] = {0, 0, 0};
+      if (table) {
+        double T[3] = {0, 0, 0};
+        if (mixed) {
+          float Ff[3] = {0, 0, 0}, Tf[3] = {0, 0, 0};
+          gather_real_f32(t, row_list(t, s), Ff, Tf);
+          for (int q = 0; q < 3; ++q) F[q] = Ff[q];
+        } else {
+          gather_real(t, row_list(t, s), F, T);
+        }
+      }
+      if (sc.walls && (fl & 0x7e)) {
+        for (int wi = 0; wi < 6; ++wi) {
+          if (!(fl & (2 << wi))) continue;
+          const double4_32a h = b.whist[wi * cap + s];
+          const int ax = wi >> 1;
+          const double sn = h.w >= 0 ? 1.0 : -1.0;
+          double F2[3] = {h.x, h.y, h.z};
+          F2[ax] += sn * fabs(h.w);
+          v[3] += 1.0;
+          v[4] += sqrt(F2[0] * F2[0] + F2[1] * F2[1] + F2[2] * F2[2]);
+          if (table)
+            for (int q = 0; q < 3; ++q) F[q] += F2[q];
+        }
+      }
+      if (!(fl & 1)) {
+        v[1] += sqrt(F[0] * F[0] + F[1] * F[1] + F[2] * F[2]);
+        v[2] += 1.0;
+      }
     }
+    block_reduce_store<5>(v, partials);
+    return;
   }
-  block_reduce_store<3>(v, partials);
-}
-
-// real sphere-sphere rows: count, sum |F|, Love-Weber stress sum F_i (x1 - x2')_j
-__global__ void k_row_stats(Table t, double *partials, int mixed) {
+  const int nrow = gridDim.x - nbody, mine = blockIdx.x - nbody;
+  const long long r0 = t.row_start[s0], r1 = t.row_start[s0 + n];
+  double *out = partials + 5 * (long long)nbody;
   double v[11] = {0};
-  for (long long k = (long long)blockIdx.x * kT + threadIdx.x; k < t.P; k += (long long)gridDim.x * kT) {
-    double4_32a f, m, n;
+  for (long long k = r0 + (long long)mine * kT + threadIdx.x; k < r1; k += (long long)nrow * kT) {
+    double4_32a f, m, h;
     if (mixed) {
       if (t.g32[k].w == 0.0f) continue;
-      const float4 a = t.oFM32[2 * k], c = t.oFM32[2 * k + 1], h = t.hn32[k];
+      const float4 a = t.oFM32[2 * k], c = t.oFM32[2 * k + 1], e = t.hn32[k];
       f = make_double4_32a(a.x, a.y, a.z, a.w);
       m = make_double4_32a(c.x, c.y, c.z, c.w);
-      n = make_double4_32a(h.x, h.y, h.z, h.w);
+      h = make_double4_32a(e.x, e.y, e.z, e.w);
     } else {
       if (t.hfs[k].w == 0.0) continue;
-      f = t.oFM[2 * k]; m = t.oFM[2 * k + 1]; n = t.hn[k];
+      f = t.oFM[2 * k]; m = t.oFM[2 * k + 1]; h = t.hn[k];
     }
     const double l = f.w + m.w;
     v[0] += 1.0;
     v[1] += sqrt(f.x * f.x + f.y * f.y + f.z * f.z);
-    const double F3[3] = {f.x, f.y, f.z}, br[3] = {-l * n.x, -l * n.y, -l * n.z};
+    const double F3[3] = {f.x, f.y, f.z}, br[3] = {-l * h.x, -l * h.y, -l * h.z};
     for (int a = 0; a < 3; ++a)
       for (int c = 0; c < 3; ++c) v[2 + 3 * a + c] += F3[a] * br[c];
   }
-  block_reduce_store<11>(v, partials);
-}
-
-// wall contacts: count, sum |F|
-__global__ void k_wall_stats(Bodies b, SceneConst sc, const Mat *__restrict__ mats, long long cap,
-                             double *partials) {
-  double v[2] = {0, 0};
-  for (long long i = (long long)blockIdx.x * kT + threadIdx.x; i < sc.N; i += (long long)gridDim.x * kT) {
-    const uint8_t fl = b.flags[i];
-    if (!(fl & 0x7e)) continue;
-    for (int wi = 0; wi < 6; ++wi) {
-      if (!(fl & (2 << wi))) continue;
-      const double4_32a h = b.whist[wi * cap + i];
-      const int ax = wi >> 1;
-      const double sn = h.w >= 0 ? 1.0 : -1.0;
-      double F2[3] = {h.x, h.y, h.z};
-      F2[ax] += sn * fabs(h.w);
-      v[0] += 1.0;
-      v[1] += sqrt(F2[0] * F2[0] + F2[1] * F2[1] + F2[2] * F2[2]);
-    }
-  }
-  block_reduce_store<2>(v, partials);
+  block_reduce_store<11>(v, out + 11 * (long long)(mine - (int)blockIdx.x));
+  if (mine == 0 && threadIdx.x == 0) out[11 * (long long)nrow] = (double)(r1 - r0);
 }
 
 inline unsigned blocks(long long n) { return (unsigned)((n + kT - 1) / kT); }
@@ -1511,25 +1531,16 @@ void launch_gather_forces(const Bodies &b, const Table &t, const Mat *mats, cons
     k_gather_forces<<<blocks(sc.N), kT, 0, st>>>(b, t, mats, cs, sc, cap, F, T, mixed);
 }
 
-int stats_blocks(long long n) {
-  long long b = (n + kT - 1) / kT;
-  return (int)(b < 1 ? 1 : (b > 1024 ? 1024 : b));
+int stats_blocks(long long n) {   // four blocks an SM of the 152-SM part at most
+  const long long b = (n + kT - 1) / kT;
+  return (int)(b < 1 ? 1 : (b > 608 ? 608 : b));
 }
 
-void launch_body_stats(const Bodies &b, const double4_32a *F, long long N, double *partials,
-                       cudaStream_t st) {
-  k_body_stats<<<stats_blocks(N), kT, 0, st>>>(b, F, N, partials);
-}
-
-void launch_row_stats(const Table &t, const Bodies &b, double *partials, int mixed,
-                      cudaStream_t st) {
-  (void)b;
-  k_row_stats<<<stats_blocks(t.P), kT, 0, st>>>(t, partials, mixed);
-}
-
-void launch_wall_stats(const Bodies &b, const SceneConst &sc, const Mat *mats, long long cap,
-                           double *partials, cudaStream_t st) {
-  k_wall_stats<<<stats_blocks(sc.N), kT, 0, st>>>(b, sc, mats, cap, partials);
+void launch_stats(const Bodies &b, const Table &t, const Mat *mats, const CellState *cs,
+                  const SceneConst &sc, long long cap, long long s0, long long n, int table,
+                  int mixed, int nbody, int nrow, double *partials, cudaStream_t st) {
+  k_stats<<<nbody + nrow, kT, 0, st>>>(b, t, mats, cs, sc, cap, s0, n, table, mixed, nbody,
+                                       partials);
 }
 
 }  // namespace dem

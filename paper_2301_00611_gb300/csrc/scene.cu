@@ -1951,14 +1951,6 @@ dem_status dem_get_timing(dem_scene *s, dem_timing *out) {
 }
 
 namespace {
-Bodies body_view(const Bodies &b, long long o) {
-  Bodies v = b;
-  auto sh = [o](auto *&p, long long k = 1) { if (p) p += k * o; };
-  sh(v.pos); sh(v.vel); sh(v.angvel); sh(v.ori); sh(v.xref); sh(v.mprop);
-  sh(v.id); sh(v.sid); sh(v.mat); sh(v.flags); sh(v.live); sh(v.wnear); sh(v.whist); sh(v.rdsc);
-  sh(v.p32); sh(v.vw32, 2); sh(v.xref32); sh(v.mprop32); sh(v.ori32);
-  return v;
-}
 Table row_view(const Table &t, long long o, long long P) {
   Table v = t;
   auto sh = [o](auto *&p) { if (p) p += o; };
@@ -1991,52 +1983,27 @@ dem_status stats_of(dem_scene *s, int q, dem_stats *o) {
            (u.cs.box_hi[2] - u.cs.box_lo[2]);
   o->packing_fraction = V > 0 ? vsolid / V : 0;
   if (nb_ == 0) return DEM_OK;
+  // one launch and one copy; blocks by the body count alone, so that a sub-scene's sums are
+  // taken in the same order as those of the scene alone
   const bool have_table = s->table_fresh;
-  const Table &t = s->tab[s->tc];
-  const SceneConst sc = scene_const(s);
-  long long r0 = 0, r1 = have_table ? t.P : 0;
-  if (q >= 0 && have_table) {   // rows whose first body is in the sub-scene
-    CK(cudaMemcpyAsync(&s->rb_h->totals[0], t.row_start + b0, sizeof(int), cudaMemcpyDeviceToHost, s->st));
-    CK(cudaMemcpyAsync(&s->rb_h->totals[1], t.row_start + b0 + nb_, sizeof(int), cudaMemcpyDeviceToHost, s->st));
-    if ((r = wait(s))) return r;
-    r0 = s->rb_h->totals[0];
-    r1 = s->rb_h->totals[1];
-  }
-  o->n_candidates = r1 - r0;
-  double *ph = s->partials_h;
-  // bodies: kinetic energy, |F| of free bodies
-  if (have_table)
-    launch_gather_forces(s->cur, t, s->mats_d, s->cs_d, sc, s->cap, s->gF, s->gT, s->mixed, s->st);
-  else CK(cudaMemsetAsync(s->gF, 0, sizeof(double4_32a) * s->N, s->st));
-  const Bodies bv = body_view(s->cur, b0);
-  int nb = stats_blocks(nb_);
-  launch_body_stats(bv, s->gF + b0, nb_, s->partials, s->st);
-  CK(cudaMemcpyAsync(ph, s->partials, sizeof(double) * 3 * nb, cudaMemcpyDeviceToHost, s->st));
+  const int nb = stats_blocks(nb_), nr = have_table ? stats_blocks(8 * nb_) : 0;
+  const size_t words = 5 * (size_t)nb + 11 * (size_t)nr + (nr ? 1 : 0);
+  launch_stats(s->cur, s->tab[s->tc], s->mats_d, s->cs_d, scene_const(s), s->cap, b0, nb_, have_table,
+               s->mixed, nb, nr, s->partials, s->st);
+  CK(cudaGetLastError());
+  CK(cudaMemcpyAsync(s->partials_h, s->partials, sizeof(double) * words, cudaMemcpyDeviceToHost, s->st));
   if ((r = wait(s))) return r;
-  double ke = 0, sumF = 0, ndyn = 0;
-  for (int b = 0; b < nb; ++b) { ke += ph[3 * b]; sumF += ph[3 * b + 1]; ndyn += ph[3 * b + 2]; }
-  double nc = 0, sumC = 0, sig[9] = {0};
-  if (have_table && r1 > r0) {
-    const Table tv = row_view(t, r0, r1 - r0);
-    int nr = stats_blocks(tv.P);
-    launch_row_stats(tv, bv, s->partials, s->mixed, s->st);
-    CK(cudaMemcpyAsync(ph, s->partials, sizeof(double) * 11 * nr, cudaMemcpyDeviceToHost, s->st));
-    if ((r = wait(s))) return r;
-    for (int b = 0; b < nr; ++b) {
-      nc += ph[11 * b];
-      sumC += ph[11 * b + 1];
-      for (int k = 0; k < 9; ++k) sig[k] += ph[11 * b + 2 + k];
-    }
+  const double *ph = s->partials_h;
+  double ke = 0, sumF = 0, ndyn = 0, nc = 0, sumC = 0, sig[9] = {0}, nw = 0, sumW = 0;
+  for (int b = 0; b < nb; ++b, ph += 5) {
+    ke += ph[0]; sumF += ph[1]; ndyn += ph[2]; nw += ph[3]; sumW += ph[4];
   }
-  double nw = 0, sumW = 0;
-  if (s->has_walls) {
-    SceneConst sv = sc;
-    sv.N = nb_;
-    launch_wall_stats(bv, sv, s->mats_d, s->cap, s->partials, s->st);
-    CK(cudaMemcpyAsync(ph, s->partials, sizeof(double) * 2 * nb, cudaMemcpyDeviceToHost, s->st));
-    if ((r = wait(s))) return r;
-    for (int b = 0; b < nb; ++b) { nw += ph[2 * b]; sumW += ph[2 * b + 1]; }
+  for (int b = 0; b < nr; ++b, ph += 11) {
+    nc += ph[0];
+    sumC += ph[1];
+    for (int k = 0; k < 9; ++k) sig[k] += ph[2 + k];
   }
+  o->n_candidates = nr ? (long long)ph[0] : 0;
   o->kinetic_energy = ke;
   o->n_contacts = (long long)nc;
   o->n_wall_contacts = (long long)nw;
