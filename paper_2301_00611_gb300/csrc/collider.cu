@@ -183,7 +183,7 @@ __global__ void k_reorder(Bodies src, Bodies dst, long long N, long long cap,
     dst.mprop32[p] = src.mprop32[o];
     dst.ori32[p] = src.ori32[o];   // the mixed path keeps the orientation in FP32
   }
-  dst.ori[p] = src.ori[o];
+  if (!mixed) dst.ori[p] = src.ori[o];
   dst.mprop[p] = src.mprop[o];
   dst.rdsc[p] = src.rdsc[o];
   dst.xref[p] = make_double4_32a(x.x, x.y, x.z, 0.0);
@@ -387,9 +387,17 @@ __device__ inline void write_row(const RowArgs &a, int r, int s, int j, const in
   if (ot.P > 0) {
     const int o1 = a.new_to_old[s], o2 = a.new_to_old[j];
     if (o1 < a.N_old && o2 < a.N_old) {
-      const int e = ot.row_start[o1 + 1];
-      for (int q = ot.row_start[o1]; q < e; ++q)
-        if (ot.pair[q].y == o2 && ot.cpack[q] == cp) { hit = q; break; }
+      // only a row that was real has a history: its bit of the last step (whole words of
+      // bits are zero for most bodies of a loose scene)
+      const int first = ot.row_start[o1], e = ot.row_start[o1 + 1];
+      for (int q0 = first; q0 < e && hit < 0; q0 += 32) {
+        unsigned m = __funnelshift_r(ot.bits[q0 >> 5], ot.bits[(q0 >> 5) + 1], q0 & 31);
+        if (e - q0 < 32) m &= (1u << (e - q0)) - 1u;
+        for (; m; m &= m - 1) {
+          const int q = q0 + __ffs(m) - 1;
+          if (ot.pair[q].y == o2 && ot.cpack[q] == cp) { hit = q; break; }
+        }
+      }
     }
   }
   const double4_32a z = make_double4_32a(0, 0, 0, 0);

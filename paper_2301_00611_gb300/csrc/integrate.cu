@@ -240,10 +240,8 @@ __global__ void __launch_bounds__(512, (kFeat & 1) ? 2 : 3) k_integrate_mixed(co
   const float dtf = (float)dt;
   float F[3] = {0, 0, 0}, T[3] = {0, 0, 0};
   const RowList rows = row_list(t, s);   // (loaded beside the flag, not after it)
-  if (b.live[s]) {   // no row of the body is real otherwise
-    b.live[s] = 0;
-    gather_real_f32(t, rows, F, T);   // fixed order, FP32 sums
-  }
+  const bool touched = b.live[s];        // no row of the body is real otherwise
+  if (touched) gather_real_f32(t, rows, F, T);   // fixed order, FP32 sums
   const float4 va = b.vw32[2 * s], vb = b.vw32[2 * s + 1];   // v-, w- in FP32
   const float4 off = b.p32[s];                                // x - xref, r
   const float4 xr = b.xref32[s];
@@ -371,7 +369,9 @@ __global__ void __launch_bounds__(512, (kFeat & 1) ? 2 : 3) k_integrate_mixed(co
   b.pos[s] = make_double4_32a(xn[0], xn[1], xn[2], p.w);
   b.vel[s] = make_double4_32a(vn_[0], vn_[1], vn_[2], 0.0);
   b.angvel[s] = make_double4_32a(wn_[0], wn_[1], wn_[2], 0.0);
+  // (byte stores come last: they may alias anything, and no load moves ahead of one)
   if (flags != b.flags[s]) b.flags[s] = flags;
+  if (touched) b.live[s] = 0;
   const float vnf[3] = {(float)vn_[0], (float)vn_[1], (float)vn_[2]};
   const float wnf[3] = {(float)wn_[0], (float)wn_[1], (float)wn_[2]};
   b.vw32[2 * s] = make_float4(vnf[0], vnf[1], vnf[2], wnf[0]);
@@ -434,10 +434,8 @@ __global__ void __launch_bounds__(512) k_integrate(const StepDesc *__restrict__ 
   const double dt = c.dt;
   double F[3] = {0, 0, 0}, T[3] = {0, 0, 0};
   const RowList rows = row_list(t, s);   // (loaded beside the flag, not after it)
-  if (b.live[s]) {   // no row of the body is real otherwise
-    b.live[s] = 0;
-    gather_real(t, rows, F, T);
-  }
+  const bool touched = b.live[s];        // no row of the body is real otherwise
+  if (touched) gather_real(t, rows, F, T);
 
   const double4_32a p = b.pos[s];
   const double4_32a v = b.vel[s];
@@ -565,7 +563,9 @@ __global__ void __launch_bounds__(512) k_integrate(const StepDesc *__restrict__ 
   b.pos[s] = make_double4_32a(xn[0], xn[1], xn[2], r);
   b.vel[s] = make_double4_32a(vn_[0], vn_[1], vn_[2], 0.0);
   b.angvel[s] = make_double4_32a(wn_[0], wn_[1], wn_[2], 0.0);
+  // (byte stores come last: they may alias anything, and no load moves ahead of one)
   if (flags != b.flags[s]) b.flags[s] = flags;
+  if (touched) b.live[s] = 0;
 
   // orientation: q+ = dq(w+ dt) q, dq = (cos x, (sin x / x) * w dt / 2), x = |w| dt / 2.
   // For x < 1e-2 the Maclaurin series of cos x and sin x / x truncated after the x^4

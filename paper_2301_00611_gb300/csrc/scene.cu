@@ -817,6 +817,8 @@ dem_status rebuild_core(dem_scene *s) {
   if (ot.P > 0) CK(cudaMemsetAsync(ot.found, 0, sizeof(int) * ot.P, s->st));
   Table otv = ot;
   if (ot.P == 0 || ot.row_start == nullptr) otv.P = 0;
+  // every row counts as real until the contact kernel says otherwise
+  CK(cudaMemsetAsync(nt.bits, 0xff, sizeof(unsigned) * (P / 32 + 2), s->st));
   launch_rows(cr, s->cur, s->grids_d, multi, s->cell_start, nt, otv, NL,
               s->tab_nbody[s->tc], s->new_to_old, cl, s->mixed, s->st);
   launch_degree_order(nt, NL, s->st);
@@ -1913,6 +1915,7 @@ dem_status dem_set_contacts(dem_scene *s, long long n, const int *id1, const int
     }
   }
   CK(cudaMemcpyAsync(t.row_start, rs.data(), sizeof(int) * (N + 1), cudaMemcpyHostToDevice, s->st));
+  CK(cudaMemsetAsync(t.bits, 0xff, sizeof(unsigned) * (P / 32 + 2), s->st));   // all are real
   t.P = P;
   s->tab_nbody[s->tc] = N;
   s->table_fresh = false;
