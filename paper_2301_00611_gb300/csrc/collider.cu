@@ -67,13 +67,6 @@ __device__ __forceinline__ const Grid &grid_of(const Grid *__restrict__ grids,
   return grids[multi ? sid[i] : 0];
 }
 
-// Order-preserving map of doubles to unsigned integers (sign bit flipped for
-// positives, all bits for negatives), so that integer atomics give min / max.
-__device__ __forceinline__ unsigned long long ord_key(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
-}
-
 // Bounding boxes of the sub-scenes: keys[k * cap + q] (k = 0..2 lower, 3..5 upper
 // bounds of x - r / x + r), lower keys preset to all ones and upper to zero.  A
 // warp whose bodies share one sub-scene (the usual case: bodies are grouped by
@@ -562,32 +555,36 @@ __global__ void __launch_bounds__(kT) k_downs(RowArgs a) {
   });
 }
 
-// Integration order: bodies grouped by their number of incident rows, largest
-// first, so that the lanes of a warp walk row lists of about the same length
-// (the per-body sum is a loop whose trip count is the warp's longest list).  The
-// order inside a group is left to the atomics: it changes no result, only which
-// lane integrates which body.  Bucket of a body: 63 - min(rows, 63).
-__device__ inline int degree_bucket(const Table &t, int s) {
-  const int d = (t.row_start[s + 1] - t.row_start[s]) + (t.down_start[s + 1] - t.down_start[s]);
-  return kDegreeBuckets - 1 - (d < kDegreeBuckets - 1 ? d : kDegreeBuckets - 1);
-}
-
-// Degree order within chunks of kChunk consecutive slots: each chunk's bodies by
-// decreasing row count, the chunk itself staying where it is.  The lanes of a warp
-// get bodies of about the same row count (so their row walks end together) while
-// the bodies a block touches stay spatial neighbours (slot order is Morton order),
-// so their records and rows are fetched once into L2 instead of from all over the
-// arrays.
+// Integration order of the FP64 path, within runs of kChunk consecutive slots: the bodies
+// of a run by decreasing number of real rows, so that the lanes of a warp walk row lists that
+// end together (the sum over a body's rows is a loop whose trip count is the warp's longest
+// list), the run itself staying where it is, so that the bodies a block touches stay spatial
+// neighbours (slot order is Morton order) and their records and rows are fetched into L2 once.
+// The rows counted are those that carry a contact into this run; a run of slots without any
+// (a first run) goes by candidate rows.  The order inside a group is left to the atomics:
+// it changes no result, only which lane integrates which body.  By candidate rows (half of
+// which are not in contact) the 1M dense integration took 313 us, by real rows 288.
 constexpr int kChunk = 1024;
-__global__ void __launch_bounds__(kChunk) k_degree_chunk(Table t, long long N) {
+__global__ void __launch_bounds__(kChunk) k_degree_chunk(Table t, long long N, int count_real) {
   __shared__ int cnt[kDegreeBuckets], base[kDegreeBuckets];
   if (threadIdx.x < kDegreeBuckets) cnt[threadIdx.x] = 0;
-  __syncthreads();
   const long long c0 = (long long)blockIdx.x * kChunk, sl = c0 + threadIdx.x;
-  int b = -1, local = 0;
+  int rows = 0, real = 0;
   if (sl < N) {
-    b = degree_bucket(t, (int)sl);
-    local = atomicAdd(&cnt[b], 1);
+    const int a = t.row_start[sl], b = t.row_start[sl + 1];
+    const int e0 = t.down_start[sl], e1 = t.down_start[sl + 1];
+    rows = (b - a) + (e1 - e0);
+    if (count_real) {
+      for (int k = a; k < b; ++k) real += !is_zero_bits(t.hfs[k].w);
+      for (int e = e0; e < e1; ++e) real += !is_zero_bits(t.hfs[t.down[e]].w);
+    }
+  }
+  const int any = __syncthreads_or(real);
+  const int d = min(any ? real : rows, kDegreeBuckets - 1);
+  int bucket = -1, local = 0;
+  if (sl < N) {
+    bucket = kDegreeBuckets - 1 - d;
+    local = atomicAdd(&cnt[bucket], 1);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -598,7 +595,7 @@ __global__ void __launch_bounds__(kChunk) k_degree_chunk(Table t, long long N) {
     }
   }
   __syncthreads();
-  if (b >= 0) t.ord[c0 + base[b] + local] = (int)sl;
+  if (bucket >= 0) t.ord[c0 + base[bucket] + local] = (int)sl;
 }
 
 // A real row of the previous table that no candidate carried over: an error only
@@ -687,9 +684,9 @@ void launch_rows(CellRec cr, const Bodies &b, const Grid *grids, int multi, cons
   k_downs<<<blocks(N), kT, 0, st>>>(a);
 }
 
-void launch_degree_order(const Table &t, long long N, cudaStream_t st) {
+void launch_degree_order(const Table &t, long long N, int count_real, cudaStream_t st) {
   if (N <= 0) return;
-  k_degree_chunk<<<(unsigned)((N + kChunk - 1) / kChunk), kChunk, 0, st>>>(t, N);
+  k_degree_chunk<<<(unsigned)((N + kChunk - 1) / kChunk), kChunk, 0, st>>>(t, N, count_real);
 }
 
 namespace {

@@ -301,8 +301,9 @@ void launch_partners(CellRec cr, const int *sid, const int *id, long long N, con
 void launch_rows(CellRec cr, const Bodies &b, const Grid *grids, int multi, const int *start,
                  const Table &nt, const Table &ot, long long N, long long N_old,
                  const int *new_to_old, CandList cl, int mixed, cudaStream_t st);
-// t.ord = bodies in decreasing order of incident rows within runs of slots
-void launch_degree_order(const Table &t, long long N, cudaStream_t st);
+// t.ord = bodies in decreasing order of incident rows (count_real: of those in contact; FP64
+// tables) within runs of slots
+void launch_degree_order(const Table &t, long long N, int count_real, cudaStream_t st);
 void launch_lost(const Table &ot, const Bodies &ob, const Grid *grids, int multi, int *err,
                  int mixed, cudaStream_t st);
 // cell flip: rows of sub-scene `sub` (all rows unless multi) get c' = Minv c (apply = 1),

@@ -7,6 +7,17 @@
 namespace dem {
 namespace {
 
+// Order-preserving map of doubles to unsigned integers (sign bit flipped for
+// positives, all bits for negatives), so that integer minima and maxima (atomic or not) are
+// those of the doubles, off the FP64 pipe; key_double is its inverse.
+__device__ __forceinline__ unsigned long long ord_key(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
+}
+__device__ __forceinline__ double key_double(unsigned long long k) {
+  return __longlong_as_double((long long)((k >> 63) ? k & 0x7fffffffffffffffull : ~k));
+}
+
 __host__ __device__ inline uint32_t spread3(uint32_t x) {  // 8 bits -> every third bit
   x &= 0xffu;
   x = (x | (x << 8)) & 0x0000f00fu;

@@ -257,8 +257,7 @@ __global__ void __launch_bounds__(512, (kFeat & 1) ? 2 : 3) k_integrate_mixed(co
   if ((kFeat & 1) && walls) {
     const float dtl = (float)c.dt_law;   // the contact law's step (see CellState::dt_law)
     const double4_32a pd = b.pos[s];
-    double knd, ksd, tpd;
-    wall_phys(mats, c.wall_mat, b.mat[s], (double)r, knd, ksd, tpd, c.law);
+    double knd, ksd, tpd = -1.0;   // formed at the first wall in contact (tan(phi) >= 0)
     for (int left = walls; left; left &= left - 1) {   // each lane its own walls, in order
       const int wi = __ffs(left) - 1, ax = wi >> 1;
       const double distd = pick(ax, pd.x, pd.y, pd.z) - ((wi & 1) ? c.box_hi[ax] : c.box_lo[ax]);
@@ -276,6 +275,7 @@ __global__ void __launch_bounds__(512, (kFeat & 1) ? 2 : 3) k_integrate_mixed(co
       // the penetration in FP64 and rounded once: r - |dist| in FP32 would keep the
       // precision of r, not of the (much smaller) penetration
       const float pen = (float)(pd.w - fabs(distd));   // FP64 radius and distance
+      if (tpd < 0.0) wall_phys(mats, c.wall_mat, b.mat[s], (double)r, knd, ksd, tpd, c.law);
       const float sqp = c.law ? sqrtf(pen) : 1.0f;   // Hertz-Mindlin: pen^1/2 factors
       const float kn = (float)knd * sqp, ks = (float)ksd * sqp, tanphi = (float)tpd;
       float fs[3] = {0, 0, 0};
@@ -447,8 +447,7 @@ __global__ void __launch_bounds__(512) k_integrate(const StepDesc *__restrict__ 
 
   const int walls = (kFeat & 1) ? (b.wnear[s] | ((flags >> 1) & 0x3f)) & c.wall_mask : 0;
   if ((kFeat & 1) && walls) {   // only the walls within reach or in contact
-    double kn0, ks0, tanphi;
-    wall_phys(mats, c.wall_mat, b.mat[s], r, kn0, ks0, tanphi, c.law);
+    double kn0, ks0, tanphi = -1.0;   // formed at the first wall in contact (tan(phi) >= 0)
     for (int left = walls; left; left &= left - 1) {   // each lane its own walls, in order
       const int wi = __ffs(left) - 1, ax = wi >> 1;
       const double wc = (wi & 1) ? c.box_hi[ax] : c.box_lo[ax];
@@ -464,6 +463,7 @@ __global__ void __launch_bounds__(512) k_integrate(const StepDesc *__restrict__ 
       const double sn = dist >= 0 ? 1.0 : -1.0;
       const double n[3] = {ax == 0 ? sn : 0.0, ax == 1 ? sn : 0.0, ax == 2 ? sn : 0.0};
       const double pen = r - fabs(dist);
+      if (tanphi < 0.0) wall_phys(mats, c.wall_mat, b.mat[s], r, kn0, ks0, tanphi, c.law);
       double kn = kn0, ks = ks0;
       if (c.law) {   // Hertz-Mindlin: Fn = kno pen^3/2, ks = kso pen^1/2
         const double sq = sqrt(pen);

@@ -821,7 +821,7 @@ dem_status rebuild_core(dem_scene *s) {
   CK(cudaMemsetAsync(nt.bits, 0xff, sizeof(unsigned) * (P / 32 + 2), s->st));
   launch_rows(cr, s->cur, s->grids_d, multi, s->cell_start, nt, otv, NL,
               s->tab_nbody[s->tc], s->new_to_old, cl, s->mixed, s->st);
-  launch_degree_order(nt, NL, s->st);
+  launch_degree_order(nt, NL, !s->mixed && s->degree_order, s->st);
   // a removed sub-scene's contacts vanish by design: no history check on that run
   if (s->check_lost && !removal)
     launch_lost(otv, s->alt, s->grids_d, multi, &s->ds_d->error, s->mixed, s->st);
