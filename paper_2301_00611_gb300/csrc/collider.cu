@@ -301,17 +301,13 @@ __global__ void __launch_bounds__(kT) k_partners_warp(CellRec cr, const int *__r
   const float4 a = cr.wpos[s];
   const int packed = cr.info[s].x;
   const int ci[3] = {packed & 1023, (packed >> 10) & 1023, (packed >> 20) & 1023};
-  const float reach = cand_reach(g);
   int first = 0, end = 0, code = kNoWrap;
   if (lane < kStencil) stencil_cell(g, start, ci, lane, first, end, code);
-  float3 at = make_float3(a.x, a.y, a.z);
-  float sh[3] = {0, 0, 0};
+  CellShift at{make_float3(a.x, a.y, a.z), make_float3(0.0f, 0.0f, 0.0f)};
   if (code != kNoWrap && end > first) {
     int w[3];
     code_wrap(code, w);
-    wrap_shift_f32(g, w, sh);
-    const float3 mv = moved_f32(sh, code);
-    at = make_float3(__fadd_rn(a.x, mv.x), __fadd_rn(a.y, mv.y), __fadd_rn(a.z, mv.z));
+    at = cell_shift(g, a, w, lane > kStencil / 2);
   }
   int n = 0;
   for (int j = first; __any_sync(all, j < end); ++j) {
@@ -319,7 +315,7 @@ __global__ void __launch_bounds__(kT) k_partners_warp(CellRec cr, const int *__r
     if (j < end) {
       const float4 p = __ldg(cr.wpos + j);
       float d2, R;
-      keep = cand_f32(at, a.w, placed_f32(p, sh, code), p.w, reach, d2, R) && j != s;
+      keep = cand_f32(g, at, a.w, p, d2, R) && j != s;
     }
     const unsigned m = __ballot_sync(all, keep);
     const int k = n + __popc(m & ((1u << lane) - 1u));

@@ -82,24 +82,29 @@ __device__ inline void wrap_shift_f32(const Grid &g, const int w[3], float sh[3]
 // Conservative FP32 candidate test of (s, j): keeps every pair whose FP64 distance is
 // below r1 + r2 + reach (the slack covers the FP32 rounding of coordinates bounded by the
 // cell size), so the candidate set is a superset of the exact one.  A pair met from both
-// sides must be decided alike, so the image shift goes to the same of the two spheres
-// from either side (to the partner of wrap code above 13; code and 26 - code are opposite
-// wraps) and every operation is written out: no contraction that differs by call site.
-__device__ inline float3 placed_f32(const float4 &b, const float sh[3], int code) {
-  return code > 13 ? make_float3(__fadd_rn(b.x, sh[0]), __fadd_rn(b.y, sh[1]), __fadd_rn(b.z, sh[2]))
-                   : make_float3(b.x, b.y, b.z);
+// sides must be decided alike, so the image shift goes to the same of the two spheres from
+// either side: to the one in the forward half of the other's stencil ((dz, dy, dx)
+// lexicographically positive), as when every pair is met from that side only.  Every
+// operation is written out: no contraction that differs by call site.
+struct CellShift {
+  float3 me, partner;   // the body's own position; what is added to the partners'
+};
+__device__ inline CellShift cell_shift(const Grid &g, const float4 &a, const int w[3], bool fwd) {
+  float sh[3];
+  wrap_shift_f32(g, w, sh);
+  if (fwd) return {make_float3(a.x, a.y, a.z), make_float3(sh[0], sh[1], sh[2])};
+  return {make_float3(__fsub_rn(a.x, sh[0]), __fsub_rn(a.y, sh[1]), __fsub_rn(a.z, sh[2])),
+          make_float3(0.0f, 0.0f, 0.0f)};
 }
-__device__ inline float3 moved_f32(const float sh[3], int code) {   // what the body itself moves by
-  return code < 13 ? make_float3(-sh[0], -sh[1], -sh[2]) : make_float3(0.0f, 0.0f, 0.0f);
-}
-__device__ inline bool cand_f32(const float3 &a, float ra, const float3 &b, float rb, float reach,
-                                float &d2, float &R) {   // a, b placed; reach = cand_reach(g)
-  const float dx = __fsub_rn(b.x, a.x), dy = __fsub_rn(b.y, a.y), dz = __fsub_rn(b.z, a.z);
-  R = __fadd_rn(__fadd_rn(ra, rb), reach);
-  d2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
+__device__ inline bool cand_f32(const Grid &g, const CellShift &at, float ra, const float4 &b,
+                                float &d2, float &R) {
+  const float dx = __fsub_rn(__fadd_rn(b.x, at.partner.x), at.me.x);
+  const float dy = __fsub_rn(__fadd_rn(b.y, at.partner.y), at.me.y);
+  const float dz = __fsub_rn(__fadd_rn(b.z, at.partner.z), at.me.z);
+  R = __fadd_rn(__fadd_rn(__fadd_rn(ra, b.w), g.reachf), g.slack);
+  d2 = __fmaf_rn(dz, dz, __fmaf_rn(dx, dx, __fmul_rn(dy, dy)));
   return d2 < __fmul_rn(R, R);
 }
-__device__ inline float cand_reach(const Grid &g) { return __fadd_rn(g.reachf, g.slack); }
 
 constexpr int kStencil = 27;
 constexpr int kNoWrap = 13;   // wrap code of no wrap at all: (w0 + 1) + 3 (w1 + 1) + 9 (w2 + 1)
@@ -155,7 +160,6 @@ __device__ inline void walk_cells(const Grid &g, const float4 *__restrict__ wpos
                                   const int *__restrict__ start, int packed, int s, F &&f) {
   constexpr int kAhead = kHalf ? 2 : 4;
   const float4 me = wpos[s];
-  const float reach = cand_reach(g);
   const int ci[3] = {packed & 1023, (packed >> 10) & 1023, (packed >> 20) & 1023};
   bool okx[3];
   int px[3], wx[3];
@@ -195,13 +199,10 @@ __device__ inline void walk_cells(const Grid &g, const float4 *__restrict__ wpos
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
         const int code = (wx[i] + 1) + 3 * (wy + 1) + 9 * (wz + 1);
-        float3 at = make_float3(me.x, me.y, me.z);
-        float sh[3] = {0, 0, 0};
+        CellShift at{make_float3(me.x, me.y, me.z), make_float3(0.0f, 0.0f, 0.0f)};
         if (code != kNoWrap) {
           const int w[3] = {wx[i], wy, wz};
-          wrap_shift_f32(g, w, sh);
-          const float3 mv = moved_f32(sh, code);
-          at = make_float3(__fadd_rn(me.x, mv.x), __fadd_rn(me.y, mv.y), __fadd_rn(me.z, mv.z));
+          at = cell_shift(g, me, w, dz > 0 || (dz == 0 && (dy > 0 || (dy == 0 && i == 2))));
         }
         for (int j = a[i]; j < b[i]; j += kAhead) {
           float4 p[kAhead];
@@ -210,7 +211,7 @@ __device__ inline void walk_cells(const Grid &g, const float4 *__restrict__ wpos
 #pragma unroll
           for (int q = 0; q < kAhead; ++q) {
             float d2, R;
-            const bool near = cand_f32(at, me.w, placed_f32(p[q], sh, code), p[q].w, reach, d2, R);
+            const bool near = cand_f32(g, at, me.w, p[q], d2, R);
             if (near && j + q < b[i] && (kHalf || j + q != s)) f(j + q, code, d2, R);
           }
         }
