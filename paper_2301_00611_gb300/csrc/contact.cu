@@ -264,7 +264,10 @@ __global__ void __launch_bounds__(kT, kT == 128 ? 6 : 2) k_contact(const StepDes
       const double R = __dadd_rn(p1.w, p2.w);
       r1 = p1.w; r2 = p2.w;
       real = lt_nonneg(l2, __dmul_rn(R, R));   // l2 < R^2
-      if (!real && !is_zero_bits(t.hfs[k].w)) {   // contact lost (u_N > 0): back to potential
+      // contact lost (u_N > 0): back to potential.  Only a row that was real in the last step
+      // (its bit; all are set by a collider run) has a history record to look at: 300k loose
+      // spheres, most of their rows apart, 100 steps 14.1 -> 13.5 ms
+      if (!real && ((t.bits[base >> 5] >> lane) & 1u) && !is_zero_bits(t.hfs[k].w)) {
         const double4_32a z = make_double4_32a(0, 0, 0, 0);
         t.hfs[k] = z; t.hn[k] = z; t.oFM[2 * k] = z; t.oFM[2 * k + 1] = z;
       }
