@@ -817,8 +817,9 @@ dem_status rebuild_core(dem_scene *s) {
   if (ot.P > 0) CK(cudaMemsetAsync(ot.found, 0, sizeof(int) * ot.P, s->st));
   Table otv = ot;
   if (ot.P == 0 || ot.row_start == nullptr) otv.P = 0;
-  // every row counts as real until the contact kernel says otherwise
-  CK(cudaMemsetAsync(nt.bits, 0xff, sizeof(unsigned) * (P / 32 + 2), s->st));
+  // every row counts as real until the contact kernel says otherwise (no candidate pair: the
+  // row arrays may not exist yet)
+  if (P > 0) CK(cudaMemsetAsync(nt.bits, 0xff, sizeof(unsigned) * (P / 32 + 2), s->st));
   launch_rows(cr, s->cur, s->grids_d, multi, s->cell_start, nt, otv, NL,
               s->tab_nbody[s->tc], s->new_to_old, cl, s->mixed, s->st);
   launch_degree_order(nt, NL, !s->mixed && s->degree_order, s->st);
