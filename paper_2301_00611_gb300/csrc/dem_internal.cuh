@@ -352,7 +352,7 @@ void launch_cell_advance(CellState *cs, int nsub, DevStatus *ds, const double *s
 // sum F_a (-l n_b)
 void launch_p3d_partials(const Table &t, const DevStatus *ds, int mixed, double *partials,
                          cudaStream_t st);
-// GlobalStiffnessTimeStepper (N > 0): per-sub-scene minimum critical step applied to the due
+// GlobalStiffnessTimeStepper: per-sub-scene minimum critical step applied to the due
 // sub-scenes' dt.  keys, est_min: nsub entries preset to +inf (double, float bits), reset by
 // the launch; est: N floats of scratch, null to compute every body in FP64
 void launch_timestepper(const Bodies &b, const Table &t, CellState *cs, int nsub, DevStatus *ds,

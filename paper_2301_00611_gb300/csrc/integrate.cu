@@ -1520,8 +1520,9 @@ void launch_timestepper(const Bodies &b, const Table &t, CellState *cs, int nsub
                         const Mat *mats, long long N, long long cap, int mixed, int multi, int walls,
                         unsigned long long *keys, unsigned *est_min, float *est, cudaStream_t st) {
   const StiffArgs a{b, t, cs, mats, N, cap, mixed, multi, walls, nsub, keys, est_min, est};
-  if (est) k_stiff_est<<<blocks(N), kT, 0, st>>>(a, ds);
-  k_stiff_exact<<<blocks(N), kT, 0, st>>>(a, ds);
+  if (est && N > 0) k_stiff_est<<<blocks(N), kT, 0, st>>>(a, ds);
+  // (no bodies left: one block, which applies the steps of due sub-scenes without contacts)
+  k_stiff_exact<<<N > 0 ? blocks(N) : 1, kT, 0, st>>>(a, ds);
 }
 
 void launch_gather_forces(const Bodies &b, const Table &t, const Mat *mats, const CellState *cs,

@@ -1416,7 +1416,7 @@ dem_status dem_step(dem_scene *s, long long nsteps) {
           launch_timestepper(s->cur, t, s->cs_d, s->nsub(), s->ds_d, s->mats_d, sc.N, s->cap,
                              s->mixed, sc.multi, sc.walls, s->dt_keys,
                              reinterpret_cast<unsigned *>(s->dt_keys + s->subs_cap), est, s->st);
-          s->launches += est ? 2 : 1;
+          s->launches += est && sc.N > 0 ? 2 : 1;
         }
         if (record) CK(cudaEventRecord(ev[6 * i + 2], s->st));
         launch_integrate(s->step_d, *s->step_h, desc, s->cs_d, s->ds_d, s->mats_d, s->mixed,

@@ -96,3 +96,33 @@ def test_served_single_sphere(pkg, mixed):
         srv.release(t)
     fall = 0.5 * np.linalg.norm(w.gravity) * (50 * 1e-5) ** 2
     assert 0.5 * fall < w.pos[0, 2] - z < 1.1 * fall
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("stepper", [False, True])
+def test_scene_emptied_by_a_removal(pkg, stepper, mixed):
+    """The step after the removal of the last bodies runs on none; the scene then takes new
+    ones, which advance as in a scene of their own."""
+    a = workloads.box_cloud(300, 61, phi=0.3, inflate=1.04, vel_scale=0.05)
+    b = workloads.scaled_deposition(200, 62, 0.4, 1e7, steps=0)
+    prec = pkg.DEM_MIXED if mixed else pkg.DEM_FP64
+    s, alone = pkg.Scene(precision=prec), pkg.Scene(precision=prec)
+    for k in (s, alone):
+        k.set_dt(1e-5)
+        if stepper:
+            k.set_timestepper(safety=0.5, interval=1, default_dt=2e-5)
+    q = s.add_workload(a, 0, dt=1e-5)
+    s.step(3)
+    s.remove_subscene(q)
+    s.step(1)
+    assert s.n == 0 and s.count_contacts() == 0 and s.stats()["n_bodies"] == 0
+    assert s.clock()[0] == 4 and s.stats()["dt"] == (2e-5 if stepper else 1e-5)
+    s.step(5)
+    assert s.clock()[0] == 9
+    for k in (s, alone):
+        k.add_workload(b, 8, dt=1e-5)
+        k.step(20)
+    x, y = s.state(force=False), alone.state(force=False)
+    assert all(np.array_equal(x[k], y[k]) for k in x)
+    s.close()
+    alone.close()
