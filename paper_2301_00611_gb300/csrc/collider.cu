@@ -219,19 +219,6 @@ __device__ inline bool shift_overflow(const CellRec &cr, int s, int j, int code)
          abs(a.w - b.w + w[2]) > kShiftMax;
 }
 
-// Counts of a body whose partners do not fit a list (k_rows and k_downs walk again for it).
-__device__ inline void count_long(const Grid &g, const CellRec &cr, const int *__restrict__ start,
-                                  const int *__restrict__ id, int s, int *cnt_up, int *cnt_down,
-                                  bool &bad) {
-  int up = 0, down = 0;
-  walk_cells<false>(g, cr.wpos, start, cr.info[s].x, s, [&](int j, int code, float, float) {
-    (id[j] > id[s] ? up : down) += 1;
-    if (g.periodic) bad |= shift_overflow(cr, s, j, code);
-  });
-  cnt_up[s] = up;
-  cnt_down[s] = down;
-}
-
 // Partners of every body, by partner id: the down partners (smaller ids), then the rows'.
 //
 // Two shapes of the same search.  A thread per body keeps the hits in a shared-memory
@@ -247,7 +234,7 @@ __global__ void __launch_bounds__(kPT) k_partners(CellRec cr, const int *__restr
                                                   const int *__restrict__ id, long long N,
                                                   const Grid *__restrict__ grids, int multi,
                                                   const int *__restrict__ start, int *cnt_up,
-                                                  int *cnt_down, int *err, CandList cl) {
+                                                  int *cnt_down, DevStatus *ds, CandList cl) {
   __shared__ unsigned ent[kCandKeep][kPT];
   __shared__ int ids[kCandKeep][kPT];
   const int tid = threadIdx.x;
@@ -255,93 +242,132 @@ __global__ void __launch_bounds__(kPT) k_partners(CellRec cr, const int *__restr
   if (sl >= N) return;
   const int s = (int)sl, me = id[s];
   const Grid &g = grid_of(grids, sid, multi, sl);
-  bool bad = false;
   int n = 0;
   walk_cells<false>(g, cr.wpos, start, cr.info[s].x, s, [&](int j, int code, float, float) {
     if (n < kCandKeep) ent[n][tid] = (unsigned)j | ((unsigned)code << 26);
     ++n;
   });
-  if (n > cl.keep) {
-    count_long(g, cr, start, id, s, cnt_up, cnt_down, bad);
-  } else {
-    for (int k = 0; k < n; ++k) {
-      const unsigned e = ent[k][tid];
-      const int j = (int)(e & 0x3ffffffu);
-      ids[k][tid] = __ldg(id + j);
-      if (g.periodic) bad |= shift_overflow(cr, s, j, (int)(e >> 26));
-    }
-    int down = 0;
-    unsigned *mine = cl.list + (long long)s * kCandKeep;
-    for (int k = 0; k < n; ++k) {
-      const int ik = ids[k][tid];
-      int rank = 0;
-      for (int q = 0; q < n; ++q) rank += ids[q][tid] < ik;
-      mine[rank] = ent[k][tid];
-      down += ik < me;
-    }
-    cnt_down[s] = down;
-    cnt_up[s] = n - down;
+  if (n > kCandKeep) {   // for k_partners_warp
+    cl.long_ids[atomicAdd(&ds->n_long, 1)] = s;
+    return;
   }
-  if (bad) atomicOr(err, kErrShiftRange);
+  bool bad = false;
+  for (int k = 0; k < n; ++k) {
+    const unsigned e = ent[k][tid];
+    const int j = (int)(e & 0x3ffffffu);
+    ids[k][tid] = __ldg(id + j);
+    if (g.periodic) bad |= shift_overflow(cr, s, j, (int)(e >> 26));
+  }
+  int down = 0;
+  unsigned *mine = cl.list + (long long)s * kCandKeep;
+  for (int k = 0; k < n; ++k) {
+    const int ik = ids[k][tid];
+    int rank = 0;
+    for (int q = 0; q < n; ++q) rank += ids[q][tid] < ik;
+    mine[rank] = ent[k][tid];
+    down += ik < me;
+  }
+  cnt_down[s] = down;
+  cnt_up[s] = n - down;
+  if (bad) atomicOr(&ds->error, kErrShiftRange);
 }
 
+// kLong: the bodies of cl.long_ids; else all N.  A list of more than a warp's lanes is
+// ranked in shared memory and written to the spill buffer, so that its body too is walked
+// once: with the lists of 32 alone, and such bodies walked four times by single threads,
+// a run over 1M dense spheres took 5.0 ms at a sweep margin of r_min (27 partners a body) and
+// 14.8 ms at 1.25 r_min (40); now 2.6 and 4.3 ms.
+template <bool kLong>
 __global__ void __launch_bounds__(kT) k_partners_warp(CellRec cr, const int *__restrict__ sid,
                                                       const int *__restrict__ id, long long N,
                                                       const Grid *__restrict__ grids, int multi,
                                                       const int *__restrict__ start, int *cnt_up,
-                                                      int *cnt_down, int *err, CandList cl) {
-  __shared__ unsigned ent[kT / 32][kCandKeep];
+                                                      int *cnt_down, DevStatus *ds, CandList cl) {
+  __shared__ unsigned ent[kT / 32][kLongKeep];
+  __shared__ int ids[kT / 32][kLongKeep];
   const unsigned all = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const long long sl = ((long long)blockIdx.x * kT + threadIdx.x) >> 5;
-  if (sl >= N) return;
   unsigned *mine = ent[threadIdx.x >> 5];
-  const int s = (int)sl, me = id[s];
-  const Grid &g = grid_of(grids, sid, multi, sl);
-  const float4 a = cr.wpos[s];
-  const int packed = cr.info[s].x;
-  const int ci[3] = {packed & 1023, (packed >> 10) & 1023, (packed >> 20) & 1023};
-  int first = 0, end = 0, code = kNoWrap;
-  if (lane < kStencil) stencil_cell(g, start, ci, lane, first, end, code);
-  CellShift at{make_float3(a.x, a.y, a.z), make_float3(0.0f, 0.0f, 0.0f)};
-  if (code != kNoWrap && end > first) {
-    int w[3];
-    code_wrap(code, w);
-    at = cell_shift(g, a, w, lane > kStencil / 2);
-  }
-  int n = 0;
-  for (int j = first; __any_sync(all, j < end); ++j) {
-    bool keep = false;
-    if (j < end) {
-      const float4 p = __ldg(cr.wpos + j);
-      float d2, R;
-      keep = cand_f32(g, at, a.w, p, d2, R) && j != s;
-    }
-    const unsigned m = __ballot_sync(all, keep);
-    const int k = n + __popc(m & ((1u << lane) - 1u));
-    if (keep && k < kCandKeep) mine[k] = (unsigned)j | ((unsigned)code << 26);
-    n += __popc(m);
-  }
-  __syncwarp();
+  int *idm = ids[threadIdx.x >> 5];
+  const long long total = kLong ? ds->n_long : N;
+  const long long stride = ((long long)gridDim.x * kT) >> 5;
   bool bad = false;
-  if (n > cl.keep) {
-    if (lane == 0) count_long(g, cr, start, id, s, cnt_up, cnt_down, bad);
-  } else {
-    const unsigned e = lane < n ? mine[lane] : 0u;
-    const int j = (int)(e & 0x3ffffffu), idj = lane < n ? __ldg(id + j) : 0x7fffffff;
-    int rank = 0;
-    for (int q = 0; q < n; ++q) rank += __shfl_sync(all, idj, q) < idj;
-    const int down = __popc(__ballot_sync(all, lane < n && idj < me));
-    if (lane < n) {
-      cl.list[(long long)s * kCandKeep + rank] = e;
-      if (g.periodic) bad = shift_overflow(cr, s, j, (int)(e >> 26));
+  for (long long at = ((long long)blockIdx.x * kT + threadIdx.x) >> 5; at < total; at += stride) {
+    const int s = kLong ? cl.long_ids[at] : (int)at, me = id[s];
+    const Grid &g = grid_of(grids, sid, multi, s);
+    const float4 a = cr.wpos[s];
+    const int packed = cr.info[s].x;
+    const int ci[3] = {packed & 1023, (packed >> 10) & 1023, (packed >> 20) & 1023};
+    int first = 0, end = 0, code = kNoWrap;
+    if (lane < kStencil) stencil_cell(g, start, ci, lane, first, end, code);
+    CellShift sh{make_float3(a.x, a.y, a.z), make_float3(0.0f, 0.0f, 0.0f)};
+    if (code != kNoWrap && end > first) {
+      int w[3];
+      code_wrap(code, w);
+      sh = cell_shift(g, a, w, lane > kStencil / 2);
+    }
+    auto near = [&](int j) {
+      float d2, R;
+      return j < end && cand_f32(g, sh, a.w, __ldg(cr.wpos + j), d2, R) && j != s;
+    };
+    int n = 0;
+    for (int j = first; __any_sync(all, j < end); ++j) {
+      const bool keep = near(j);
+      const unsigned m = __ballot_sync(all, keep);
+      const int k = n + __popc(m & ((1u << lane) - 1u));
+      if (keep && k < kLongKeep) mine[k] = (unsigned)j | ((unsigned)code << 26);
+      n += __popc(m);
+    }
+    __syncwarp();
+    int down = 0;
+    if (n <= cl.keep) {
+      const unsigned e = lane < n ? mine[lane] : 0u;
+      const int j = (int)(e & 0x3ffffffu), idj = lane < n ? __ldg(id + j) : 0x7fffffff;
+      int rank = 0;
+      for (int q = 0; q < n; ++q) rank += __shfl_sync(all, idj, q) < idj;
+      down = __popc(__ballot_sync(all, lane < n && idj < me));
+      if (lane < n) {
+        cl.list[(long long)s * kCandKeep + rank] = e;
+        if (g.periodic) bad |= shift_overflow(cr, s, j, (int)(e >> 26));
+      }
+    } else if (cl.keep > 0 && n <= kLongKeep) {
+      unsigned place = 0;
+      if (lane == 0) place = atomicAdd(&ds->long_total, (unsigned)n);
+      place = __shfl_sync(all, place, 0);
+      const bool fits = (unsigned)n <= cl.spill_cap && place <= cl.spill_cap - (unsigned)n;
+      for (int k = lane; k < n; k += 32) {
+        const unsigned e = mine[k];
+        const int j = (int)(e & 0x3ffffffu), idj = __ldg(id + j);
+        idm[k] = idj;
+        down += idj < me;
+        if (g.periodic) bad |= shift_overflow(cr, s, j, (int)(e >> 26));
+      }
+      down = __reduce_add_sync(all, down);
+      __syncwarp();
+      if (fits)
+        for (int k = lane; k < n; k += 32) {
+          const int ik = idm[k];
+          int rank = 0;
+          for (int q = 0; q < n; ++q) rank += idm[q] < ik;
+          cl.spill[place + rank] = mine[k];
+        }
+      if (lane == 0) cl.list[(long long)s * kCandKeep] = fits ? place : kNoList;
+    } else {   // no list: the counts alone
+      for (int j = first; j < end; ++j) {
+        if (!near(j)) continue;
+        down += __ldg(id + j) < me;
+        if (g.periodic) bad |= shift_overflow(cr, s, j, code);
+      }
+      down = __reduce_add_sync(all, down);
+      if (lane == 0 && cl.keep > 0) cl.list[(long long)s * kCandKeep] = kNoList;
     }
     if (lane == 0) {
       cnt_down[s] = down;
       cnt_up[s] = n - down;
     }
+    __syncwarp();
   }
-  if (bad) atomicOr(err, kErrShiftRange);
+  if (bad) atomicOr(&ds->error, kErrShiftRange);
 }
 
 // What the row passes read: the walk's records and lists, the bodies in slot order, the
@@ -457,6 +483,16 @@ __device__ inline int range_of(int lo, int r) {
   return q;
 }
 
+// Where the list of body s with n partners is: kListed (its part of cl.list), its place in
+// the spill buffer, or kNoList.
+__device__ inline unsigned list_place(const CandList &cl, long long s, int n) {
+  if (n <= cl.keep) return kListed;
+  return cl.keep > 0 ? cl.list[s * kCandKeep] : kNoList;
+}
+__device__ inline unsigned list_entry(const CandList &cl, int s, unsigned place, int k) {
+  return place == kListed ? cl.list[(long long)s * kCandKeep + k] : cl.spill[(size_t)place + k];
+}
+
 // Rows, 32 at a time: a warp takes 32 bodies, whose rows are consecutive, so every store
 // to the new table is coalesced whatever the bodies' row counts.
 __global__ void __launch_bounds__(kT) k_rows(RowArgs a) {
@@ -467,23 +503,23 @@ __global__ void __launch_bounds__(kT) k_rows(RowArgs a) {
   const long long me = base + lane < a.N ? base + lane : a.N;
   const int lo = a.t.row_start[me], hi = me < a.N ? a.t.row_start[me + 1] : lo;
   const int nd = me < a.N ? a.t.down_start[me + 1] - a.t.down_start[me] : 0;
-  const bool listed = nd + hi - lo <= a.cl.keep;
+  const unsigned place = list_place(a.cl, me, nd + hi - lo);
   const int end = __shfl_sync(all, hi, 31);
   for (int r0 = __shfl_sync(all, lo, 0); r0 < end; r0 += 32) {
     const int r = r0 + lane;
     const int q = range_of(lo, r);
     const int from = __shfl_sync(all, lo, q), skip = __shfl_sync(all, nd, q);
-    const bool mine = __shfl_sync(all, (int)listed, q);
-    if (r < end && mine) {
+    const unsigned mine = __shfl_sync(all, place, q);
+    if (r < end && mine != kNoList) {
       const int s = (int)base + q;
-      const unsigned e = a.cl.list[(long long)s * kCandKeep + skip + (r - from)];
+      const unsigned e = list_entry(a.cl, s, mine, skip + (r - from));
       int w[3];
       code_wrap((int)(e >> 26), w);
       write_row(a, r, s, (int)(e & 0x3ffffffu), w);
     }
   }
-  if (listed) return;
-  // more partners than a list holds: walk again, by insertion in order of id (found: the
+  if (place != kNoList) return;
+  // no list: walk again, by insertion in order of id (found: the
   // partner's id until the row is complete; cpack: its wrap)
   const int s = (int)me, ids = a.b.id[s];
   const Grid &g = grid_of(a.grids, a.b.sid, a.multi, s);
@@ -525,20 +561,20 @@ __global__ void __launch_bounds__(kT) k_downs(RowArgs a) {
   const long long me = base + lane < a.N ? base + lane : a.N;
   const int lo = a.t.down_start[me], hi = me < a.N ? a.t.down_start[me + 1] : lo;
   const int nu = me < a.N ? a.t.row_start[me + 1] - a.t.row_start[me] : 0;
-  const bool listed = nu + hi - lo <= a.cl.keep;
+  const unsigned place = list_place(a.cl, me, nu + hi - lo);
   const int end = __shfl_sync(all, hi, 31);
   for (int e0 = __shfl_sync(all, lo, 0); e0 < end; e0 += 32) {
     const int e = e0 + lane;
     const int q = range_of(lo, e);
     const int from = __shfl_sync(all, lo, q);
-    const bool mine = __shfl_sync(all, (int)listed, q);
-    if (e < end && mine) {
+    const unsigned mine = __shfl_sync(all, place, q);
+    if (e < end && mine != kNoList) {
       const int s = (int)base + q;
-      const int p = (int)(a.cl.list[(long long)s * kCandKeep + (e - from)] & 0x3ffffffu);
+      const int p = (int)(list_entry(a.cl, s, mine, e - from) & 0x3ffffffu);
       a.t.down[e] = row_of(a.t, p, s);
     }
   }
-  if (listed) return;
+  if (place != kNoList) return;
   const int s = (int)me, ids = a.b.id[s];
   const Grid &g = grid_of(a.grids, a.b.sid, a.multi, s);
   int k = lo;
@@ -660,15 +696,19 @@ void launch_reorder(const Bodies &src, const Bodies &dst, long long N, long long
 }
 
 void launch_partners(CellRec cr, const int *sid, const int *id, long long N, const Grid *grids,
-                     int multi, const int *start, int *cnt_up, int *cnt_down, int *err, CandList cl,
-                     cudaStream_t st) {
+                     int multi, const int *start, int *cnt_up, int *cnt_down, DevStatus *ds,
+                     CandList cl, bool long_lists, bool again, int nsm, cudaStream_t st) {
   if (N <= 0) return;
-  if (N < kWarpBodies)
-    k_partners_warp<<<blocks(32 * N), kT, 0, st>>>(cr, sid, id, N, grids, multi, start, cnt_up,
-                                                   cnt_down, err, cl);
-  else
+  if (N < kWarpBodies || long_lists || cl.keep == 0) {
+    k_partners_warp<false><<<blocks(32 * N), kT, 0, st>>>(cr, sid, id, N, grids, multi, start,
+                                                          cnt_up, cnt_down, ds, cl);
+    return;
+  }
+  if (!again)
     k_partners<<<(unsigned)((N + kPT - 1) / kPT), kPT, 0, st>>>(cr, sid, id, N, grids, multi, start,
-                                                               cnt_up, cnt_down, err, cl);
+                                                               cnt_up, cnt_down, ds, cl);
+  k_partners_warp<true><<<7 * nsm, kT, 0, st>>>(cr, sid, id, N, grids, multi, start, cnt_up,
+                                                cnt_down, ds, cl);
 }
 
 void launch_rows(CellRec cr, const Bodies &b, const Grid *grids, int multi, const int *start,

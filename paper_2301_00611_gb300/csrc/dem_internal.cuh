@@ -181,6 +181,8 @@ struct DevStatus {
   int pending;    // collider run needed before the next step (steps are skipped)
   int request;    // set by the integrator when a displacement exceeds the bound
   int error;      // kErr* bits
+  int n_long;             // bodies of the collider run with more than kCandKeep partners,
+  unsigned long_total;    // and the entries of their lists
   int arrive;     // blocks of the current cell-advance launch that have finished
   unsigned long long steps;   // steps completed (never reset)
 };
@@ -283,19 +285,27 @@ void launch_reorder(const Bodies &src, const Bodies &dst, long long N, long long
 // per-sub-scene bounding boxes as ordered keys (see collider.cu); keys preset
 void launch_bbox_sub(const Bodies &b, long long N, int cap, unsigned long long *keys, int nsm,
                      cudaStream_t st);
-// Partners of a body, up to kCandKeep (slot and the wrap of the partner's cell, packed in
-// 32 bits), by id: those of smaller id, then those of larger id.  keep: kCandKeep, or 0
-// where slots do not fit 26 bits; a body with more partners has no list and is walked
-// again by the row passes.
-constexpr int kCandKeep = 32;
+// Partners of a body (slot and the wrap of the partner's cell, packed in 32 bits), by id:
+// those of smaller id, then those of larger id.  Up to kCandKeep have their place in `list`;
+// a longer list goes to `spill`, its place there in the first word of the body's part of
+// `list` (kNoList: it did not fit, or has more than kLongKeep entries; the row passes walk
+// again for such a body).  keep: kCandKeep, or 0 where slots do not fit 26 bits: no lists at
+// all.
+constexpr int kCandKeep = 32, kLongKeep = 512;
+constexpr unsigned kNoList = 0xffffffffu, kListed = 0xfffffffeu;
 struct CandList {
   unsigned *list;
   int keep;
+  unsigned *spill;
+  unsigned spill_cap;
+  int *long_ids;     // scratch: the bodies with more than kCandKeep (N)
 };
-// cnt_up / cnt_down: partners of larger / smaller id of every body
+// cnt_up / cnt_down: partners of larger / smaller id of every body; ds: its error word and
+// the (zeroed) counters of long lists.  long_lists: most bodies are expected to have one.
+// again: a second call for the same bodies with more room in spill (long_total zeroed)
 void launch_partners(CellRec cr, const int *sid, const int *id, long long N, const Grid *grids,
-                     int multi, const int *start, int *cnt_up, int *cnt_down, int *err, CandList cl,
-                     cudaStream_t st);
+                     int multi, const int *start, int *cnt_up, int *cnt_down, DevStatus *ds,
+                     CandList cl, bool long_lists, bool again, int nsm, cudaStream_t st);
 // rows (with the history of the old table: `found` marks the rows carried over) and down
 // lists of the new table, whose row_start and down_start are set
 void launch_rows(CellRec cr, const Bodies &b, const Grid *grids, int multi, const int *start,

@@ -13,6 +13,7 @@
 #include <chrono>
 #include <map>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -212,6 +213,8 @@ struct dem_scene {
   float4 *wpos = nullptr;
   int4 *cinfo = nullptr;
   unsigned *cand_list = nullptr;   // partners of each body (kCandKeep per body)
+  unsigned *spill = nullptr;       // lists of the bodies with more (as many as runs needed)
+  unsigned spill_cap = 0;
 
   Table tab[2]{};
   long long tab_nbody[2]{0, 0};
@@ -694,6 +697,12 @@ dem_status sub_grid(dem_scene *s, Sub &u, const double lo[3], const double hi[3]
   return DEM_OK;
 }
 
+// Mean partners of a body in the last table above which the collider takes a warp per body in
+// scenes of any size: then most bodies have a long list, and the thread-per-body pass only
+// finds that out.  A run over 1M dense spheres with a warp per body against both passes: 2.96
+// against 2.62 ms at a mean of 27, 4.34 against 5.43 at 40.
+constexpr long long kLongMean = kCandKeep;
+
 dem_status rebuild_core(dem_scene *s) {
   const long long N = s->N;   // slots in use: live bodies and those of removed sub-scenes
   const int nsub = s->nsub();
@@ -732,6 +741,7 @@ dem_status rebuild_core(dem_scene *s) {
   //    row-major for sub-scenes), consecutive in sub-scene order; bodies of removed
   //    sub-scenes take the sentinel cell after the last one
   long long total = 0, n_live = 0;
+  double partners_est = 0;   // of all bodies: number density times the volume within reach
   bool removal = false;
   for (int q = 0; q < nsub; ++q) {
     Sub &u = s->subs[q];
@@ -747,6 +757,11 @@ dem_status rebuild_core(dem_scene *s) {
     total += multi ? (long long)g.n[0] * g.n[1] * g.n[2] : (long long)g.B * g.B * g.B;
     u.slot0 = n_live;
     n_live += u.n;
+    double V = u.cs.periodic ? std::fabs(m_det(u.cs.H)) : 1.0;
+    if (!u.cs.periodic)
+      for (int k = 0; k < 3; ++k) V *= g.n[k] / g.scale[k];
+    const double reach = 2 * std::cbrt(u.vsolid / (double)u.n) + 2 * 1.612 * u.cs.verlet;
+    partners_est += (double)u.n * ((double)u.n / V) * reach * reach * reach;
   }
   if (total + 1 > 0x7fffffffLL) return fail(s, DEM_ERR_CAPACITY, "collider grid exceeds 2^31 cells");
   const uint32_t dead = (uint32_t)total;
@@ -765,7 +780,9 @@ dem_status rebuild_core(dem_scene *s) {
     }
   }
   CK(cudaMemsetAsync(s->cell_count, 0, sizeof(int) * ncell, s->st));
-  CK(cudaMemsetAsync(&s->ds_d->error, 0, sizeof(int), s->st));
+  // error word and the counters of long lists
+  static_assert(offsetof(DevStatus, long_total) == offsetof(DevStatus, error) + 2 * sizeof(int), "");
+  CK(cudaMemsetAsync(&s->ds_d->error, 0, 3 * sizeof(int), s->st));
   // ids close up over removed sub-scenes: each live sub-scene's ids move down by the
   // bodies of removed sub-scenes with smaller ids
   const int *id_shift = nullptr;
@@ -799,9 +816,24 @@ dem_status rebuild_core(dem_scene *s) {
   Table &nt = s->tab[1 - s->tc];
   if ((r = ensure_table(s, nt, 0, NL))) return r;
   // slots are packed in 26 bits of a list entry
-  const CandList cl{s->cand_list, s->cap < (1LL << 26) ? kCandKeep : 0};
-  launch_partners(cr, s->cur.sid, s->cur.id, NL, s->grids_d, multi, s->cell_start, s->cnt_up,
-                  s->cnt_down, &s->ds_d->error, cl, s->st);
+  CandList cl{s->cand_list, s->cap < (1LL << 26) ? kCandKeep : 0, s->spill, s->spill_cap,
+              reinterpret_cast<int *>(s->key)};
+  // partners to expect: those of the last table, on a first run the estimate (dense spheres of
+  // one size: 14 for 13 at the default margin, 41 for 40 at 1.25 r_min); a first buffer of the
+  // size that they would need saves the second call below
+  const double mean = ot.P > 0 ? 2.0 * ot.P / std::max<long long>(s->tab_nbody[s->tc], 1)
+                               : partners_est / std::max<long long>(NL, 1);
+  const bool long_lists = mean > kLongMean;
+  if (long_lists && !s->spill && cl.keep > 0) {
+    const long long room = (long long)std::min(1.25 * mean * NL, 268435456.0);
+    if (!dalloc(s, &s->spill, room)) s->spill_cap = cl.spill_cap = (unsigned)room;
+    cl.spill = s->spill;
+  }
+  auto partners = [&](bool again) {
+    launch_partners(cr, s->cur.sid, s->cur.id, NL, s->grids_d, multi, s->cell_start, s->cnt_up,
+                    s->cnt_down, s->ds_d, cl, long_lists, again, s->nsm, s->st);
+  };
+  partners(false);
   exclusive_scan2(s->cnt_up, nt.row_start, s->cnt_down, nt.down_start, NL, s->scan_ws, s->st);
   CK(cudaMemcpyAsync(&s->rb_h->totals[0], nt.row_start + NL, sizeof(int), cudaMemcpyDeviceToHost, s->st));
   CK(cudaMemcpyAsync(&s->rb_h->totals[1], nt.down_start + NL, sizeof(int), cudaMemcpyDeviceToHost, s->st));
@@ -812,6 +844,20 @@ dem_status rebuild_core(dem_scene *s) {
   if (P != s->rb_h->totals[1]) return fail(s, DEM_ERR_STATE, "internal: candidate count mismatch");
   if ((r = ensure_table(s, nt, P, NL))) return r;
   nt.P = P;
+  // long lists that had no room: once more with a larger buffer (without the memory for it,
+  // the row passes walk again for them)
+  const long long need = s->rb_h->ds.long_total;
+  if (need > s->spill_cap) {
+    const long long room = std::min<long long>(need + need / 4, kListed - 1);
+    unsigned *buf = nullptr;
+    if (!dalloc(s, &buf, room)) {
+      dfree(s, s->spill);
+      s->spill = cl.spill = buf;
+      s->spill_cap = cl.spill_cap = (unsigned)room;
+      CK(cudaMemsetAsync(&s->ds_d->long_total, 0, sizeof(unsigned), s->st));
+      partners(true);
+    }
+  }
   // 5-6: rows with the contact history of the previous table, down lists
   ot.P = std::min(ot.P, ot.cap);
   if (ot.P > 0) CK(cudaMemsetAsync(ot.found, 0, sizeof(int) * ot.P, s->st));
@@ -1078,7 +1124,7 @@ void dem_scene_destroy(dem_scene *s) {
   free_table(s, s->tab[1]);
   dfree(s, s->slot_of_id); dfree(s, s->new_to_old); dfree(s, s->cnt_up); dfree(s, s->cnt_down);
   dfree(s, s->key); dfree(s, s->gF); dfree(s, s->gT); dfree(s, s->wpos); dfree(s, s->cinfo);
-  dfree(s, s->cand_list);
+  dfree(s, s->cand_list); dfree(s, s->spill);
   dfree(s, s->cell_count); dfree(s, s->cell_start);
   dfree(s, s->scan_ws); dfree(s, s->partials); dfree(s, s->servo); dfree(s, s->p3d_d); dfree(s, s->p3d_part); dfree(s, s->deg_ws);
   dfree(s, s->mats_d); dfree(s, s->cs_d); dfree(s, s->ds_d);
