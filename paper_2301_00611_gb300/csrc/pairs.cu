@@ -25,6 +25,7 @@
 
 #include "dem_internal.cuh"
 #include "grid.cuh"
+#include "pinned_words.h"
 #include "dem.h"
 
 namespace dem {
@@ -432,46 +433,17 @@ dem_status read_extent(const double ext[8], double lo[3], double hi[3], double *
   return DEM_OK;
 }
 
-// Pinned words that a query's results are copied to, kept between calls (a few per
-// process: one for each call under way): a copy into pageable memory stages through the
-// driver and returns only when it is done, and a stream synchronization makes the
-// default memory pool give its freed memory back, which the next call's scratch pays
-// for.  A slot whose call timed out is not used again (the GPU may still write to it).
-class PinnedWords {
- public:
-  double *take() {
-    {
-      std::lock_guard<std::mutex> l(mu_);
-      if (!free_.empty()) {
-        double *p = free_.back();
-        free_.pop_back();
-        return p;
-      }
-    }
-    void *p = nullptr;
-    if (cudaHostAlloc(&p, 128, cudaHostAllocPortable) != cudaSuccess) {
+// Words for the results of the queries under way: a copy into pageable memory stages
+// through the driver and returns only when it is done, and a stream synchronization makes
+// the default memory pool give its freed memory back, which the next call's scratch pays for.
+PinnedWords g_pinned(
+    [](size_t bytes) -> void * {
+      void *p = nullptr;
+      if (cudaHostAlloc(&p, bytes, cudaHostAllocPortable) == cudaSuccess) return p;
       cudaGetLastError();
       return nullptr;
-    }
-    return (double *)p;
-  }
-  void give(double *p) {
-    if (!p) return;
-    {
-      std::lock_guard<std::mutex> l(mu_);
-      if (free_.size() < 16) {
-        free_.push_back(p);
-        return;
-      }
-    }
-    cudaFreeHost(p);
-  }
-
- private:
-  std::mutex mu_;
-  std::vector<double *> free_;
-};
-PinnedWords g_pinned;
+    },
+    [](void *p) { cudaFreeHost(p); });
 
 }  // namespace dem
 
@@ -499,25 +471,33 @@ extern "C" dem_status dem_find_pairs(const double *pos_dev, const double *radius
   set_global_error("");
   if (n < 2) return DEM_OK;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  double *host = g_pinned.take();
+  PinnedLease pinned(g_pinned);
   char *mem = nullptr, *mem2 = nullptr;
-  bool to = false;
   auto done = [&](dem_status c, const std::string &m) {
     if (mem2) cudaFreeAsync(mem2, st);
     if (mem) cudaFreeAsync(mem, st);
-    if (!to) g_pinned.give(host);
     return c == DEM_OK ? c : fail(c, m);
   };
   // bounded wait for `bytes` copied from the device to the pinned words
   auto fetch = [&](const void *src, size_t bytes) -> dem_status {
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(host, src, bytes, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = bounded_wait(st, &to);
+    bool to = false;
+    if (e == cudaSuccess &&
+        pinned.fetch(
+            [&] {
+              e = cudaMemcpyAsync(pinned.words(), src, bytes, cudaMemcpyDeviceToHost, st);
+              return e == cudaSuccess;
+            },
+            [&] {
+              e = bounded_wait(st, &to);
+              return e == cudaSuccess && !to;
+            }))
+      return DEM_OK;
     if (to) { err = "timed out waiting for the GPU"; return DEM_ERR_TIMEOUT; }
-    if (e != cudaSuccess) { err = std::string("pair query: ") + cudaGetErrorString(e); return DEM_ERR_CUDA; }
-    return DEM_OK;
+    err = std::string("pair query: ") + cudaGetErrorString(e);
+    return DEM_ERR_CUDA;
   };
-  if (!host) return done(DEM_ERR_OOM, "pinned host allocation failed");
+  if (!pinned.words()) return done(DEM_ERR_OOM, "pinned host allocation failed");
   // phase 1: extent
   PairScratch S{};
   if (cudaMallocAsync((void **)&mem, carve_extent(nullptr, n, S), st) != cudaSuccess) {
@@ -529,7 +509,7 @@ extern "C" dem_status dem_find_pairs(const double *pos_dev, const double *radius
   pairs_extent(pos_dev, radius_dev, n, S, st);
   double lo[3], hi[3], rmax = 0;
   dem_status r = fetch(S.ext, 8 * sizeof(double));
-  if (!r) r = read_extent(host, lo, hi, &rmax, err);
+  if (!r) r = read_extent(pinned.words(), lo, hi, &rmax, err);
   Grid g;
   if (!r) r = pair_grid(periodic, cell_h, lo, hi, rmax, margin, g, err);
   if (r) return done(r, err);
@@ -546,7 +526,7 @@ extern "C" dem_status dem_find_pairs(const double *pos_dev, const double *radius
   if (e != cudaSuccess) return done(DEM_ERR_CUDA, std::string("pair query: ") + cudaGetErrorString(e));
   if ((r = fetch(S.off + n, sizeof(int)))) return done(r, err);
   int tot = 0;
-  std::memcpy(&tot, host, sizeof tot);
+  std::memcpy(&tot, pinned.words(), sizeof tot);
   *count = tot;
   return done(DEM_OK, "");
 }
