@@ -49,14 +49,17 @@ __global__ void __launch_bounds__(kT) k_extent(const double *__restrict__ pos,
   for (long long i = (long long)blockIdx.x * kT + threadIdx.x; i < n; i += (long long)gridDim.x * kT) {
     const double x[3] = {pos[3 * i], pos[3 * i + 1], pos[3 * i + 2]}, r = rad[i];
     const long long rb = __double_as_longlong(r);
-    bad |= rb <= 0 || (rb >> 52) == 0x7ff;   // not positive, infinite or NaN
+    bad |= rb <= 0;   // not positive (NaN, infinity: below)
+    unsigned e = (unsigned)(rb >> 52);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      bad |= ((__double_as_longlong(x[k]) >> 52) & 0x7ff) == 0x7ff;
+      e = max(e, (unsigned)(__double_as_longlong(x[k]) >> 52) & 0x7ff);
       const unsigned long long key = ord_key(x[k]);
       v[k] = min(v[k], key);
       v[3 + k] = max(v[3 + k], key);
     }
+    // x + y + z + r must be finite; it is where every magnitude is below 2^1022
+    if (e >= 0x7fd) bad |= !isfinite(x[0] + x[1] + x[2] + r);
     v[6] = max(v[6], (unsigned long long)rb);
   }
   if (bad) atomicOr(&ctl[0], 1);
