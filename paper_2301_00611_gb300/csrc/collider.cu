@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(kPT) k_partners(CellRec cr, const int *__restr
     if (n < kCandKeep) ent[n][tid] = (unsigned)j | ((unsigned)code << 26);
     ++n;
   });
-  if (n > kCandKeep) {   // for k_partners_warp
+  if (n > kCandKeep) {   // for k_partners_warp (no others can exceed cl.many: N < 2^26)
     cl.long_ids[atomicAdd(&ds->n_long, 1)] = s;
     return;
   }
@@ -364,6 +364,7 @@ __global__ void __launch_bounds__(kT) k_partners_warp(CellRec cr, const int *__r
     if (lane == 0) {
       cnt_down[s] = down;
       cnt_up[s] = n - down;
+      if (n > cl.many) atomicAdd(&ds->many_total, (unsigned long long)n);
     }
     __syncwarp();
   }

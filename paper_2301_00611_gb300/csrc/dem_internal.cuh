@@ -183,6 +183,7 @@ struct DevStatus {
   int error;      // kErr* bits
   int n_long;             // bodies of the collider run with more than kCandKeep partners,
   unsigned long_total;    // and the entries of their lists
+  unsigned long long many_total;   // partners of the bodies with more than partners_many(N)
   int arrive;     // blocks of the current cell-advance launch that have finished
   unsigned long long steps;   // steps completed (never reset)
 };
@@ -285,6 +286,11 @@ void launch_reorder(const Bodies &src, const Bodies &dst, long long N, long long
 // per-sub-scene bounding boxes as ordered keys (see collider.cu); keys preset
 void launch_bbox_sub(const Bodies &b, long long N, int cap, unsigned long long *keys, int nsm,
                      cudaStream_t st);
+// The row counts are summed in 32 bits.  Bodies with more partners than this are added up in
+// 64 bits as well (many_total); the others have 2^31 together at most, so the sum of all is
+// known: many_total <= 2 P < many_total + 2^31, with P modulo 2^32 from the prefix sum.  No
+// body of an ordinary scene has as many (a million bodies: 2147).
+inline long long partners_many(long long N) { return (1LL << 31) / (N > 0 ? N : 1); }
 // Partners of a body (slot and the wrap of the partner's cell, packed in 32 bits), by id:
 // those of smaller id, then those of larger id.  Up to kCandKeep have their place in `list`;
 // a longer list goes to `spill`, its place there in the first word of the body's part of
@@ -299,9 +305,10 @@ struct CandList {
   unsigned *spill;
   unsigned spill_cap;
   int *long_ids;     // scratch: the bodies with more than kCandKeep (N)
+  long long many;    // partners_many(N)
 };
 // cnt_up / cnt_down: partners of larger / smaller id of every body; ds: its error word and
-// the (zeroed) counters of long lists.  long_lists: most bodies are expected to have one.
+// the (zeroed) counters of partners and long lists.  long_lists: most bodies are expected to have one.
 // again: a second call for the same bodies with more room in spill (long_total zeroed)
 void launch_partners(CellRec cr, const int *sid, const int *id, long long N, const Grid *grids,
                      int multi, const int *start, int *cnt_up, int *cnt_down, DevStatus *ds,

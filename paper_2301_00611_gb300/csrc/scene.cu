@@ -780,9 +780,9 @@ dem_status rebuild_core(dem_scene *s) {
     }
   }
   CK(cudaMemsetAsync(s->cell_count, 0, sizeof(int) * ncell, s->st));
-  // error word and the counters of long lists
-  static_assert(offsetof(DevStatus, long_total) == offsetof(DevStatus, error) + 2 * sizeof(int), "");
-  CK(cudaMemsetAsync(&s->ds_d->error, 0, 3 * sizeof(int), s->st));
+  // error word and the counters of the run
+  constexpr size_t counters = offsetof(DevStatus, arrive) - offsetof(DevStatus, error);
+  CK(cudaMemsetAsync(&s->ds_d->error, 0, counters, s->st));
   // ids close up over removed sub-scenes: each live sub-scene's ids move down by the
   // bodies of removed sub-scenes with smaller ids
   const int *id_shift = nullptr;
@@ -817,7 +817,7 @@ dem_status rebuild_core(dem_scene *s) {
   if ((r = ensure_table(s, nt, 0, NL))) return r;
   // slots are packed in 26 bits of a list entry
   CandList cl{s->cand_list, s->cap < (1LL << 26) ? kCandKeep : 0, s->spill, s->spill_cap,
-              reinterpret_cast<int *>(s->key)};
+              reinterpret_cast<int *>(s->key), partners_many(NL)};
   // partners to expect: those of the last table, on a first run the estimate (dense spheres of
   // one size: 14 for 13 at the default margin, 41 for 40 at 1.25 r_min); a first buffer of the
   // size that they would need saves the second call below
@@ -841,6 +841,11 @@ dem_status rebuild_core(dem_scene *s) {
   if ((r = wait(s))) return r;
   if (s->rb_h->ds.error) return status_error(s, s->rb_h->ds.error);
   const long long P = s->rb_h->totals[0];
+  // the number of pairs beyond 32 bits (see partners_many)
+  const unsigned long long many = s->rb_h->ds.many_total, half = many / 2;
+  const unsigned long long pairs = half + (unsigned)((unsigned)P - (unsigned)half);
+  if (pairs > 0x7fffffffULL)
+    return fail(s, DEM_ERR_CAPACITY, "more than 2^31-1 candidate pairs (sweep margin or overlaps too large)");
   if (P != s->rb_h->totals[1]) return fail(s, DEM_ERR_STATE, "internal: candidate count mismatch");
   if ((r = ensure_table(s, nt, P, NL))) return r;
   nt.P = P;

@@ -77,3 +77,18 @@ def test_trajectory_does_not_depend_on_the_margin(env, n):
         s.close()
     for other in out[1:]:
         assert all(np.array_equal(a, b) for a, b in zip(out[0], other))
+
+
+@pytest.mark.parametrize("n", [65537, 92683])
+def test_more_candidate_pairs_than_a_table_can_hold(env, n):
+    """Every pair within the margin: n (n - 1) / 2 is just above 2^31 and just above 2^32, where
+    a 32-bit sum comes out negative and small.  Both are an error, not a table."""
+    torch, pkg = env
+    s = pkg.Scene(box_hi=(1, 1, 1), verlet_dist=10.0)
+    s.set_material(0, 2600.0, 1e7, 0.3, 0.5)
+    s.add_spheres(workloads.uniform(3 * n, 31).reshape(n, 3), np.full(n, 1e-6))
+    s.set_dt(1e-9)
+    with pytest.raises(pkg.DemError) as e:
+        s.step(1)
+    assert e.value.code == 4 and "pairs" in str(e.value)
+    s.close()
