@@ -631,8 +631,8 @@ dem_status dem_get_body_stress(dem_scene *scene, double *out);
  * found them), the same on every call.  Scratch memory is allocated on
  * cuda_stream (NULL: the default stream) and freed before returning; the call
  * waits for its work.  Errors (reported by dem_last_error(NULL)): INVALID_ARG,
- * NONFINITE, GEOMETRY (a sphere pair spans a third of the periodic cell), OOM,
- * TIMEOUT, CUDA. */
+ * NONFINITE, GEOMETRY (a sphere pair spans a third of the periodic cell), CAPACITY
+ * (more than 2^32-1 pairs), OOM, TIMEOUT, CUDA. */
 dem_status dem_find_pairs(const double *pos_dev, const double *radius_dev, long long n,
                           int periodic, const double *cell_h, double margin, long long cap,
                           int *id1_dev, int *id2_dev, int *cell_dist_dev, long long *count,

@@ -35,13 +35,23 @@ constexpr int kT = 256;
 
 inline unsigned blocks(long long n) { return (unsigned)((n + kT - 1) / kT); }
 
+// Counters of a query, zeroed at its start.
+struct PairCtl {
+  int bad, blocks;            // extent pass: bad input, blocks done
+  // The pairs are summed in 32 bits.  Spheres with more pairs than `many` (2^31 / n) are added
+  // up in 64 bits as well; the others have 2^31 pairs together at most, so the sum of
+  // all is known: big <= pairs < big + 2^31, `low` the pairs modulo 2^32.
+  unsigned long long big;
+  unsigned low;
+};
+
 // extent of the configuration: min x, max x per axis and max r per block, as ordered keys; the
 // last block to finish reduces the partials to ext[0..6] and sets ext[7] to 1 for bad input.
-// ctl: two zeroed ints (bad input, blocks done).  In FP64 the comparisons alone kept the
+// ctl: zeroed (bad input, blocks done).  In FP64 the comparisons alone kept the
 // FP64 pipe busy: 62 us for a million spheres, 18 us for 3001 (now 23 and 8).
 __global__ void __launch_bounds__(kT) k_extent(const double *__restrict__ pos,
                                                const double *__restrict__ rad, long long n,
-                                               unsigned long long *partials, int *ctl, double *ext) {
+                                               unsigned long long *partials, PairCtl *ctl, double *ext) {
   __shared__ unsigned long long sh[7][kT / 32];
   __shared__ int last;
   unsigned long long v[7] = {~0ull, ~0ull, ~0ull, 0, 0, 0, 0};
@@ -62,7 +72,7 @@ __global__ void __launch_bounds__(kT) k_extent(const double *__restrict__ pos,
     if (e >= 0x7fd) bad |= !isfinite(x[0] + x[1] + x[2] + r);
     v[6] = max(v[6], (unsigned long long)rb);
   }
-  if (bad) atomicOr(&ctl[0], 1);
+  if (bad) atomicOr(&ctl->bad, 1);
   auto reduce = [&]() {   // v of thread 0: the block's
 #pragma unroll
     for (int q = 0; q < 7; ++q) {
@@ -83,7 +93,7 @@ __global__ void __launch_bounds__(kT) k_extent(const double *__restrict__ pos,
   if (threadIdx.x == 0) {
     for (int q = 0; q < 7; ++q) partials[7 * blockIdx.x + q] = v[q];
     __threadfence();
-    last = atomicAdd(&ctl[1], 1) == (int)gridDim.x - 1;
+    last = atomicAdd(&ctl->blocks, 1) == (int)gridDim.x - 1;
   }
   __syncthreads();
   if (!last) return;
@@ -98,7 +108,7 @@ __global__ void __launch_bounds__(kT) k_extent(const double *__restrict__ pos,
   if (threadIdx.x == 0) {
     for (int q = 0; q < 6; ++q) ext[q] = key_double(v[q]);
     ext[6] = __longlong_as_double((long long)v[6]);
-    ext[7] = *(volatile int *)&ctl[0];
+    ext[7] = *(volatile int *)&ctl->bad;
   }
 }
 
@@ -209,7 +219,7 @@ constexpr long long kPairSlots = 1LL << 26;
 // Count pass, a thread per slot.  A million spheres at solid fraction 0.62, whole query:
 // 4.15 -> 0.53 ms; 3001 spheres: 0.35 -> 0.16 ms.
 __global__ void __launch_bounds__(kT) k_pair_count(PairView v, Grid g, unsigned *list, int keep,
-                                                   int *cnt) {
+                                                   long long many, int *cnt, PairCtl *ctl) {
   const long long sl = (long long)blockIdx.x * kT + threadIdx.x;
   if (sl >= v.n) return;
   const int s = (int)sl;
@@ -223,6 +233,7 @@ __global__ void __launch_bounds__(kT) k_pair_count(PairView v, Grid g, unsigned 
     ++n;
   });
   cnt[s] = n;
+  if (n > many) atomicAdd(&ctl->big, (unsigned long long)n);
 }
 
 struct PairOut {
@@ -245,43 +256,46 @@ __device__ inline void put_pair(const PairView &v, const Grid &g, const PairOut 
 
 // Rows of the pairs: a warp takes 32 slots, whose rows are consecutive, and writes 32 rows
 // at a time from the lists; a slot with more pairs than its list holds walks its cells again.
+// Offsets are unsigned (up to 2^32 - 1 pairs), those within a warp's rows relative to its first.
 __global__ void __launch_bounds__(kT) k_pair_emit(PairView v, Grid g, const unsigned *__restrict__ list,
-                                                  int keep, const int *__restrict__ off, PairOut o) {
+                                                  int keep, const unsigned *__restrict__ off,
+                                                  PairCtl *ctl, PairOut o) {
   const unsigned all = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const long long base = ((long long)blockIdx.x * kT + threadIdx.x) & ~31LL;
   if (base >= v.n) return;
   const long long me = base + lane < v.n ? base + lane : v.n;
-  const int lo = off[me], hi = off[me < v.n ? me + 1 : v.n];
-  const bool listed = hi - lo <= keep;
-  const int end = __shfl_sync(all, hi, 31);
-  for (int r0 = __shfl_sync(all, lo, 0); r0 < end; r0 += 32) {
-    const int r = r0 + lane;
+  const unsigned at = off[me], to = off[me < v.n ? me + 1 : v.n];
+  const bool listed = to - at <= (unsigned)keep;
+  const unsigned begin = __shfl_sync(all, at, 0), lo = at - begin, end = __shfl_sync(all, to, 31) - begin;
+  for (unsigned r0 = 0; r0 < end; r0 += 32) {
+    const unsigned r = r0 + lane;
     int q = 0;   // the last slot whose rows begin at or before r
 #pragma unroll
     for (int step = 16; step > 0; step >>= 1) {
-      const int b = __shfl_sync(all, lo, q + step);
+      const unsigned b = __shfl_sync(all, lo, q + step);
       if (b <= r) q += step;
     }
-    const int from = __shfl_sync(all, lo, q);
+    const unsigned from = __shfl_sync(all, lo, q);
     const bool mine = __shfl_sync(all, (int)listed, q);
     if (r < end && mine) {
       const int s = (int)base + q;
       const unsigned e = list[(long long)s * kPairKeep + (r - from)];
       int w[3];
       code_wrap((int)(e >> 26), w);
-      put_pair(v, g, o, r, s, (int)(e & 0x3ffffffu), w);
+      put_pair(v, g, o, (long long)begin + r, s, (int)(e & 0x3ffffffu), w);
     }
   }
   if (!listed) {
     const int s = (int)me;
-    long long r = lo;
+    long long r = at;
     walk_cells<true>(g, v.cr.wpos, v.start, v.cr.info[s].x, s, [&](int j, int code, float d2, float R) {
       int w[3];
       code_wrap(code, w);
       if (is_pair(v, g, s, j, w, d2, R)) put_pair(v, g, o, r++, s, j, w);
     });
   }
+  if (me == v.n - 1) ctl->low = to;
 }
 
 double now_s() {
@@ -357,7 +371,7 @@ dem_status pair_grid(int periodic, const double *H, const double lo[3], const do
 struct PairScratch {
   unsigned long long *partials;
   double *ext;
-  int *ctl;                  // bad input, blocks done
+  PairCtl *ctl;
   uint32_t *key;
   int *count, *start, *tmp, *order, *cnt, *off, *ws;
   CellRec raw, cr;
@@ -374,7 +388,7 @@ int extent_blocks(long long n) {
 size_t carve_extent(char *base, long long n, PairScratch &s) {
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
   char *p = base;
-  s.ctl = (int *)p; p += 256;
+  s.ctl = (PairCtl *)p; p += 256;
   s.ext = (double *)p; p += 256;
   s.partials = (unsigned long long *)p; p += up(8 * 7 * extent_blocks(n));
   return (size_t)(p - base);
@@ -402,11 +416,11 @@ size_t carve_grid(char *base, long long n, long long ncell, PairScratch &s) {
 // First phase of a query: the extent of the inputs, into S.ext (device).
 void pairs_extent(const double *pos, const double *rad, long long n, const PairScratch &S,
                   cudaStream_t st) {
-  cudaMemsetAsync(S.ctl, 0, 2 * sizeof(int), st);
+  cudaMemsetAsync(S.ctl, 0, sizeof(PairCtl), st);
   k_extent<<<extent_blocks(n), kT, 0, st>>>(pos, rad, n, S.partials, S.ctl, S.ext);
 }
 
-// Second phase: bin, sort, count, scan, emit; the pair count ends up in S.off[n].
+// Second phase: bin, sort, count, scan, emit; the pair count ends up in S.ctl.
 cudaError_t pairs_launch(const double *pos, const double *rad, long long n, const Grid &g,
                          double margin, const PairScratch &S, long long cap, int *I, int *J, int *C,
                          cudaStream_t st) {
@@ -418,10 +432,22 @@ cudaError_t pairs_launch(const double *pos, const double *rad, long long n, cons
   k_place<<<blocks(n), kT, 0, st>>>(n, S.tmp, S.key, S.start, S.raw, S.order, S.cr);
   const PairView v{pos, rad, S.order, S.cr, S.start, margin, n};
   const int keep = n <= kPairSlots ? kPairKeep : 0;
-  k_pair_count<<<blocks(n), kT, 0, st>>>(v, g, S.list, keep, S.cnt);
+  k_pair_count<<<blocks(n), kT, 0, st>>>(v, g, S.list, keep, (1LL << 31) / n, S.cnt, S.ctl);
   exclusive_scan(S.cnt, S.off, n, S.ws, st);
-  k_pair_emit<<<blocks(n), kT, 0, st>>>(v, g, S.list, keep, S.off, PairOut{cap, I, J, C});
+  k_pair_emit<<<blocks(n), kT, 0, st>>>(v, g, S.list, keep, (const unsigned *)S.off, S.ctl,
+                                        PairOut{cap, I, J, C});
   return cudaGetLastError();
+}
+
+// The pair count as the host reads it.
+dem_status read_count(const PairCtl &ctl, long long *count, std::string &err) {
+  const unsigned long long total = ctl.big + (ctl.low - (unsigned)ctl.big);
+  if (total > 0xffffffffULL) {
+    err = "more than 2^32-1 pairs";
+    return DEM_ERR_CAPACITY;
+  }
+  *count = (long long)total;
+  return DEM_OK;
 }
 
 // The extent as the host reads it: errors of the inputs, box and largest radius.
@@ -527,11 +553,11 @@ extern "C" dem_status dem_find_pairs(const double *pos_dev, const double *radius
   const cudaError_t e = pairs_launch(pos_dev, radius_dev, n, g, margin, S, cap, id1_dev, id2_dev,
                                      cell_dist_dev, st);
   if (e != cudaSuccess) return done(DEM_ERR_CUDA, std::string("pair query: ") + cudaGetErrorString(e));
-  if ((r = fetch(S.off + n, sizeof(int)))) return done(r, err);
-  int tot = 0;
-  std::memcpy(&tot, pinned.words(), sizeof tot);
-  *count = tot;
-  return done(DEM_OK, "");
+  PairCtl ctl;
+  if ((r = fetch(S.ctl, sizeof ctl))) return done(r, err);
+  std::memcpy(&ctl, pinned.words(), sizeof ctl);
+  r = read_count(ctl, count, err);
+  return done(r, err);
 }
 
 // ---------------------------------------------------------------------------
@@ -654,8 +680,8 @@ extern "C" dem_status dem_find_pairs_noalloc(const double *pos_dev, const double
   if (pairs_launch(pos_dev, radius_dev, n, g, margin, S, cap, id1_dev, id2_dev, cell_dist_dev,
                    st) != cudaSuccess)
     return fail(DEM_ERR_CUDA, "pair query launch failed");
-  int tot = 0;
-  if ((r = fetch(&tot, S.off + n, sizeof tot))) return fail(r, err);
-  *count = tot;
+  PairCtl ctl;
+  if ((r = fetch(&ctl, S.ctl, sizeof ctl))) return fail(r, err);
+  if ((r = read_count(ctl, count, err))) return fail(r, err);
   return DEM_OK;
 }

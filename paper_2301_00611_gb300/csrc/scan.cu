@@ -7,7 +7,8 @@
 // tile needs the second launch only.  More than kMaxDirect tiles (16.8M items): the
 // tile sums are scanned first, by the same two launches.
 // Two arrays of the same length can share the launches (grid y).
-// out has n + 1 entries: out[n] is the total.  Deterministic (integers).
+// out has n + 1 entries: out[n] is the total.  Deterministic (integers; sums are modulo 2^32,
+// and the callers whose totals can exceed that check them).
 //
 // The five launches this replaced (tile scan, scan of the sums with its total, add,
 // total) took 2.0-5.8 us each on a GB300 for 1M items, most of it launch latency.
@@ -27,13 +28,13 @@ struct ScanArgs {
   int *sums[2];        // tile sums, or (scanned) their exclusive prefix sums
 };
 
-__device__ inline int block_sum(int v) {
-  __shared__ int part[kThreads / 32];
+__device__ inline unsigned block_sum(unsigned v) {
+  __shared__ unsigned part[kThreads / 32];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
   __syncthreads();
-  int s = 0;
+  unsigned s = 0;
 #pragma unroll
   for (int w = 0; w < kThreads / 32; ++w) s += part[w];
   return s;
@@ -42,20 +43,20 @@ __device__ inline int block_sum(int v) {
 __global__ void __launch_bounds__(kThreads) k_tile_sums(ScanArgs a, long long n) {
   const int *__restrict__ in = a.in[blockIdx.y];
   const long long base = (long long)blockIdx.x * kTile;
-  int s = 0;
+  unsigned s = 0;
 #pragma unroll
   for (int i = 0; i < kItems; ++i) {
     const long long g = base + i * kThreads + threadIdx.x;
     s += g < n ? in[g] : 0;
   }
   s = block_sum(s);
-  if (threadIdx.x == 0) a.sums[blockIdx.y][blockIdx.x] = s;
+  if (threadIdx.x == 0) a.sums[blockIdx.y][blockIdx.x] = (int)s;
 }
 
 // scanned: a.sums already holds the exclusive prefix of the tile sums
 __global__ void __launch_bounds__(kThreads) k_scan_tiles(ScanArgs a, long long n, int scanned) {
-  __shared__ int tile[kTile];
-  __shared__ int warp_tot[kThreads / 32];
+  __shared__ unsigned tile[kTile];
+  __shared__ unsigned warp_tot[kThreads / 32];
   const int *__restrict__ in = a.in[blockIdx.y];
   int *__restrict__ out = a.out[blockIdx.y];
   const int *__restrict__ sums = a.sums[blockIdx.y];
@@ -66,7 +67,7 @@ __global__ void __launch_bounds__(kThreads) k_scan_tiles(ScanArgs a, long long n
     const long long g = base + i * kThreads + t;
     tile[i * kThreads + t] = (g < n) ? in[g] : 0;
   }
-  int before = 0;   // items of the tiles before this one
+  unsigned before = 0;   // items of the tiles before this one
   if (scanned) {
     before = sums[blockIdx.x];
   } else if (blockIdx.x > 0) {
@@ -74,8 +75,8 @@ __global__ void __launch_bounds__(kThreads) k_scan_tiles(ScanArgs a, long long n
     before = block_sum(before);
   }
   __syncthreads();
-  int v[kItems];
-  int run = 0;
+  unsigned v[kItems];
+  unsigned run = 0;
 #pragma unroll
   for (int i = 0; i < kItems; ++i) {
     v[i] = run;
@@ -83,24 +84,24 @@ __global__ void __launch_bounds__(kThreads) k_scan_tiles(ScanArgs a, long long n
   }
   // inclusive warp scan of the per-thread totals
   const int lane = t & 31, wid = t >> 5;
-  int x = run;
+  unsigned x = run;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    int y = __shfl_up_sync(0xffffffffu, x, o);
+    unsigned y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
   if (lane == 31) warp_tot[wid] = x;
   __syncthreads();
-  int off = before + (x - run);
+  unsigned off = before + (x - run);
   for (int w = 0; w < wid; ++w) off += warp_tot[w];
 #pragma unroll
   for (int i = 0; i < kItems; ++i) tile[t * kItems + i] = v[i] + off;
-  if (t == kThreads - 1 && base + kTile >= n) out[n] = off + run;
+  if (t == kThreads - 1 && base + kTile >= n) out[n] = (int)(off + run);
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < kItems; ++i) {
     const long long g = base + i * kThreads + t;
-    if (g < n) out[g] = tile[i * kThreads + t];
+    if (g < n) out[g] = (int)tile[i * kThreads + t];
   }
 }
 
