@@ -505,11 +505,15 @@ const char *dem_server_last_error(dem_server *server);
  * section 3.1.6; this library exposes the GPU launch geometry instead.)
  *   contact_block          threads per block of the contact kernel: 128 or 256
  *   contact_blocks_per_sm  blocks per SM of the contact kernel's persistent grid,
- *                          1..64 (each warp walks rows/(SMs*blocks*block/32) rows)
+ *                          1..64 (each warp walks rows/(SMs*blocks*block/32) rows).
+ *                          At most as many are launched as an SM holds at a time: FP64
+ *                          6 of 128 threads or 2 of 256, mixed precision 8 or 4; any
+ *                          larger value launches that many
  *   integrate_block        threads per block of the integrator: 128, 256 or 512
  *   degree_order           1: integrate the bodies of each run of 1024 slots in
- *                          decreasing order of incident contact rows (lanes of a warp
- *                          get similar row counts, a block's bodies stay neighbours);
+ *                          decreasing order of their rows in contact (mixed: of all
+ *                          their rows), so that lanes of a warp get similar row counts
+ *                          and a block's bodies stay neighbours;
  *                          0: in slot order
  *   step_graphs            1: a batch of steps is captured once as a CUDA graph and
  *                          replayed (one launch per batch; the kernels then read
@@ -521,7 +525,9 @@ const char *dem_server_last_error(dem_server *server);
  *                          -1: graphs below 262,144 bodies, where launch overhead
  *                          matters.  Batches with per-kernel timing, the stress servo
  *                          or the time stepper are never captured.
- * Defaults: 256, 8, 256, 1, -1. */
+ * A kernel over too few rows or bodies to give every SM four such blocks is launched in
+ * smaller ones (down to 32 threads).
+ * Defaults: 256, 8 (as many as an SM holds), 256, 1 (mixed precision: 0), -1. */
 typedef struct dem_tuning {
     int contact_block;
     int contact_blocks_per_sm;
@@ -535,7 +541,8 @@ dem_status dem_set_tuning(dem_scene *scene, const dem_tuning *tuning);
 dem_status dem_get_tuning(const dem_scene *scene, dem_tuning *tuning);
 
 /* Pick the launch shapes by timing the scene's own steps: six contact-kernel
- * shapes (block 128/256 x 4/8/16 blocks of 256 threads per SM), each timed twice in
+ * shapes (a quarter, half, three quarters and all of the 128-thread blocks an SM holds;
+ * half and all of the 256-thread ones), each timed twice in
  * two passes and taken per table row processed (a scene that gains contacts during
  * the trials does not favour the shapes tried first), then five more integrator
  * shapes (block 128/256/512 x body order) with the best contact shape (step_graphs is

@@ -313,12 +313,7 @@ void launch_contact(const StepDesc *d, const StepDesc &h, bool desc, long long r
   const int regs = block;   // which register budget: that of the tuned block
   block = spread_block(rows, block, nsm);
   long long need = (rows + block - 1) / block;
-  // Persistent grid: at most the blocks an SM holds at a time (see the launch bounds).  Every
-  // further block repeats the start-up and ends with its own partly filled pass of the law:
-  // two blocks of 256 an SM instead of eight, 300k loose spheres 72 -> 47 us, 100k dense
-  // Hertz-Mindlin 106 -> 94, 1M dense 548 -> 538.
-  const int resident = regs == 128 && block == 128 ? 6 : 2 * (256 / block);
-  const long long cap = (long long)nsm * (per_sm < resident ? per_sm : resident);
+  const long long cap = contact_grid(regs, block, per_sm, 0, nsm);   // persistent grid
   unsigned grid = (unsigned)(need < cap ? need : cap);
 #define DEM_C(B, F, D) k_contact<B, F, D><<<grid, block, 0, st>>>(d, h.t, h.b, cs, ds, mats, multi)
 #define DEM_CB(F, D) if (regs == 128 && block == 128) DEM_C(128, F, D); else DEM_C(256, F, D);

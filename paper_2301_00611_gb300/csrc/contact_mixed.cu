@@ -270,12 +270,7 @@ void launch_contact_mixed(const StepDesc *d, const StepDesc &h, bool desc, long 
   const int regs = block;   // which register budget: that of the tuned block
   block = spread_block(rows, block, nsm);
   long long need = (rows + block - 1) / block;
-  // Persistent grid: at most the blocks an SM holds at a time.  Further ones repeat the
-  // start-up and end with a partly filled pass of the law for each of their warps: four
-  // blocks of 256 an SM instead of eight, 1M dense spheres 148 -> 140 us, 789k in 64 loose
-  // scenes 45 -> 40 (three an SM: 163 and 45).
-  const int resident = 1024 / block;
-  const long long cap = (long long)nsm * (per_sm < resident ? per_sm : resident);
+  const long long cap = contact_grid(regs, block, per_sm, 1, nsm);   // persistent grid
   unsigned grid = (unsigned)(need < cap ? need : cap);
 #define DEM_C(B, F, D) k_contact_mixed<B, F, D><<<grid, block, 0, st>>>(d, h.t, h.b, cs, ds, mats, multi)
 #define DEM_CB(F, D) if (regs == 128 && block == 128) DEM_C(128, F, D); else DEM_C(256, F, D);

@@ -329,7 +329,7 @@ void launch_flip_shift(const Table &t, const int *sid, int multi, int sub, const
                        int *maxabs, int apply, cudaStream_t st);
 
 // contact.cu
-// block: 128 or 256 threads; per_sm: blocks per SM of the persistent grid
+// block: 128 or 256 threads; per_sm: blocks per SM of the persistent grid (see contact_grid)
 // multi: cs is an array indexed by Bodies::sid (else cs[0] holds the one scene)
 // rows: upper bound of the table rows (sizes the grid: the table capacity, so that the
 // launch shape does not change between collider runs)
@@ -354,6 +354,22 @@ inline int spread_block(long long n, int tuned, int nsm) {
   int b = tuned;
   while (b > 32 && n < 4LL * nsm * b) b = b > 128 ? 128 : b / 2;
   return b;
+}
+
+// Blocks of `tuned` threads of the contact kernels that an SM holds at a time (their launch
+// bounds), and the blocks an SM of the persistent grid when spread_block made them `block`
+// threads: per_sm of the tuned ones or as many as it holds, with as many threads.  More than
+// it holds would only repeat the start-up and end with a partly filled pass of the law each:
+// FP64, two blocks of 256 instead of eight: 300k loose spheres 72 -> 47 us, 100k dense
+// Hertz-Mindlin 106 -> 94, 1M dense 548 -> 538; mixed, four instead of eight: 1M dense 148 ->
+// 140, 789k in 64 loose scenes 45 -> 40 (three: 163 and 45).  (Blocks of 32 and
+// 64 threads, of small scenes, stay below that bound: spread_block leaves eight an SM at most.)
+inline int contact_resident(int tuned, int mixed) {
+  return mixed ? 1024 / tuned : (tuned == 128 ? 6 : 2);
+}
+inline long long contact_grid(int tuned, int block, int per_sm, int mixed, int nsm) {
+  const int held = contact_resident(tuned, mixed);
+  return (long long)nsm * (per_sm < held ? per_sm : held) * (tuned / block);
 }
 
 // integrate.cu

@@ -2148,20 +2148,23 @@ dem_status dem_autotune(dem_scene *s, long long steps, dem_tuning *chosen) {
   };
   dem_tuning best = current_tuning(s);
   double best_cost = INFINITY;
-  const int cblocks[2] = {128, 256};
-  const int per_sm[3] = {4, 8, 16};
-  double shape_cost[2][3];
+  // a quarter, half, three quarters and all of the blocks of 128 threads an SM holds; half and
+  // all of those of 256
+  struct Shape { int block, per_sm; } shapes[6];
+  const int r128 = contact_resident(128, s->mixed), r256 = contact_resident(256, s->mixed);
+  for (int k = 0; k < 4; ++k) shapes[k] = {128, (r128 * (k + 1) + 3) / 4};
+  for (int k = 0; k < 2; ++k) shapes[4 + k] = {256, (r256 * (k + 1) + 1) / 2};
+  double shape_cost[6];
   for (int pass = 0; pass < 2; ++pass)
-    for (int ib = 0; ib < 2; ++ib)
-      for (int ip = 0; ip < 3; ++ip) {
-        dem_tuning t = current_tuning(s);
-        t.contact_block = cblocks[ib];
-        t.contact_blocks_per_sm = per_sm[ip] * (256 / cblocks[ib]);
-        double c;
-        if ((r = trial(t, c))) return r;
-        shape_cost[ib][ip] = pass ? std::min(shape_cost[ib][ip], c) : c;
-        if (pass && shape_cost[ib][ip] < best_cost) { best_cost = shape_cost[ib][ip]; best = t; }
-      }
+    for (int k = 0; k < 6; ++k) {
+      dem_tuning t = current_tuning(s);
+      t.contact_block = shapes[k].block;
+      t.contact_blocks_per_sm = shapes[k].per_sm;
+      double c;
+      if ((r = trial(t, c))) return r;
+      shape_cost[k] = pass ? std::min(shape_cost[k], c) : c;
+      if (pass && shape_cost[k] < best_cost) { best_cost = shape_cost[k]; best = t; }
+    }
   const int iblocks[3] = {128, 256, 512};
   const dem_tuning base = best;
   for (int b : iblocks)
