@@ -1240,9 +1240,11 @@ inline unsigned blocks(long long n) { return (unsigned)((n + kT - 1) / kT); }
 // instructions of the FP64 pipe.  So a first pass estimates every body's ratio in FP32
 // (k_stiff_est) and takes the smallest estimate of each sub-scene; the second
 // (k_stiff_exact) computes in FP64 the bodies whose estimate is within kEstBand of it.  The
-// estimate is a sum of non-negative terms (relative error below 1e-5: the band is wide),
-// provided ks is not many times kn: materials with a ks/kn ratio above one, bodies
-// that a wall may touch, density-scaled sub-scenes and estimates outside FP32's normal
+// estimate takes the largest of three axis sums of stiffnesses that are not negative, which
+// is at least a third of their sum over the axes, so its relative error is that of the terms,
+// some 1e-6 whatever the ratio ks/kn (the band is wide).  Negative ones could cancel: scenes
+// with a Poisson's ratio above 1 (1 - nu^2 < 0) or with such contacts set by the caller, and
+// bodies that a wall may touch, density-scaled sub-scenes and estimates outside FP32's normal
 // range are computed in FP64 without one.  The last block of the second pass applies the
 // new step.  100k spheres, Hertz-Mindlin, sheared cell: 230 + 11 us -> 30 + 24 us.
 constexpr float kEstBand = 1.001f;

@@ -199,6 +199,7 @@ struct dem_scene {
   Mat mats_h[kMaxMat]{};
   bool mat_set[kMaxMat]{};
   double max_poisson = 0;        // of every material ever set
+  bool negative_phys = false;    // a contact was set with a negative stiffness
   Mat *mats_d = nullptr;
 
   long long N = 0, cap = 0;
@@ -1445,8 +1446,9 @@ dem_status dem_step(dem_scene *s, long long nsteps) {
         if (u.used && u.cs.tstep && (u.cs.iter + i) % u.cs.tstep_interval == 0) return true;
       return false;
     };
-    // the stepper's FP32 estimates (in the force buffer, which queries use) need ks <= kn
-    float *est = s->max_poisson <= 1.0 ? reinterpret_cast<float *>(s->gT) : nullptr;
+    // the stepper's FP32 estimates (in the force buffer, which queries use) need stiffnesses
+    // that are not negative: Poisson's ratios up to 1, and no others set by the caller
+    float *est = s->max_poisson <= 1.0 && !s->negative_phys ? reinterpret_cast<float *>(s->gT) : nullptr;
     // captured batches read the descriptor; launched ones take the arrays as parameters
     const bool use_graph = (s->step_graphs > 0 || (s->step_graphs < 0 && sc.N < kGraphAutoBodies)) &&
                            !ev && !servo && !tstep && !p3d;
@@ -1916,6 +1918,7 @@ dem_status dem_set_contacts(dem_scene *s, long long n, const int *id1, const int
       flags[sl] |= (2 << w);
       continue;
     }
+    s->negative_phys |= ph[0] < 0 || ph[1] < 0;
     // rows are oriented by id (body 1 = id1 < id2), as the collider orients them
     const int a = sid[id1[k]], b = sid[id2[k]];
     int c[3] = {0, 0, 0};
