@@ -103,7 +103,8 @@ struct Table {
   int *row_start;   // [nbody + 1]
   int *down_start;  // [nbody + 1]
   int *down;        // [cap]
-  int *ord;         // [nbody]: bodies by decreasing number of incident rows (integration order)
+  int *ord;         // [nbody]: integration order, within runs of 1024 slots by decreasing number of
+                    // rows in contact (mixed precision: of rows)
   int *found;       // [cap]
   long long cap;    // rows
   long long nbody_cap;
@@ -174,7 +175,7 @@ struct P3d {
 };
 
 constexpr int kServoBlocks = 304;   // fixed partial count of the controller reductions
-constexpr int kDegreeBuckets = 64;  // incident-row counts >= 63 share the last bucket
+constexpr int kDegreeBuckets = 64;  // row counts >= 63 share the last bucket
 
 // Small status block read back by the host after a batch of steps.
 struct DevStatus {
@@ -432,8 +433,8 @@ void launch_body_stress(const Bodies &b, const Table &t, long long N, long long 
 int stats_blocks(long long n);
 // bodies [s0, s0 + n) on nbody blocks and, with a table, the rows they own on nrow blocks:
 // 5 nbody + 11 nrow partials, then (nrow > 0) the number of rows
-void launch_stats(const Bodies &b, const Table &t, const Mat *mats, const CellState *cs,
-                  const SceneConst &sc, long long cap, long long s0, long long n, int table,
-                  int mixed, int nbody, int nrow, double *partials, cudaStream_t st);
+void launch_stats(const Bodies &b, const Table &t, const SceneConst &sc, long long cap, long long s0,
+                  long long n, int table, int mixed, int nbody, int nrow, double *partials,
+                  cudaStream_t st);
 
 }  // namespace dem

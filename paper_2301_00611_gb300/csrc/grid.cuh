@@ -60,12 +60,6 @@ __device__ inline void cell_of(const Grid &g, double x, double y, double z, int 
   }
 }
 
-__device__ inline int neg_shift(int p) {
-  int a, b, c;
-  unpack_shift(p, a, b, c);
-  return pack_shift(-a, -b, -c);
-}
-
 // Image shift of the cells of wrap w, in FP32 (H w of a sheared cell): the shift of -w is
 // its exact negative.
 __device__ inline void wrap_shift_f32(const Grid &g, const int w[3], float sh[3]) {

@@ -1154,10 +1154,9 @@ __device__ inline void block_reduce_store(double (&v)[K], double *partials) {
 // Separate passes (forces of every body to memory, body sums, row sums, wall sums, a copy and
 // a wait after each) cost a look at a small scene three round trips: 20k spheres 81 -> 49 us,
 // 1M dense 586 -> 396.
-__global__ void __launch_bounds__(kT) k_stats(Bodies b, Table t, const Mat *__restrict__ mats,
-                                              const CellState *__restrict__ cs, SceneConst sc,
-                                              long long cap, long long s0, long long n, int table,
-                                              int mixed, int nbody, double *partials) {
+__global__ void __launch_bounds__(kT) k_stats(Bodies b, Table t, SceneConst sc, long long cap,
+                                              long long s0, long long n, int table, int mixed,
+                                              int nbody, double *partials) {
   if ((int)blockIdx.x < nbody) {
     double v[5] = {0, 0, 0, 0, 0};
     for (long long i = (long long)blockIdx.x * kT + threadIdx.x; i < n; i += (long long)nbody * kT) {
@@ -1539,11 +1538,10 @@ int stats_blocks(long long n) {   // four blocks an SM of the 152-SM part at mos
   return (int)(b < 1 ? 1 : (b > 608 ? 608 : b));
 }
 
-void launch_stats(const Bodies &b, const Table &t, const Mat *mats, const CellState *cs,
-                  const SceneConst &sc, long long cap, long long s0, long long n, int table,
-                  int mixed, int nbody, int nrow, double *partials, cudaStream_t st) {
-  k_stats<<<nbody + nrow, kT, 0, st>>>(b, t, mats, cs, sc, cap, s0, n, table, mixed, nbody,
-                                       partials);
+void launch_stats(const Bodies &b, const Table &t, const SceneConst &sc, long long cap, long long s0,
+                  long long n, int table, int mixed, int nbody, int nrow, double *partials,
+                  cudaStream_t st) {
+  k_stats<<<nbody + nrow, kT, 0, st>>>(b, t, sc, cap, s0, n, table, mixed, nbody, partials);
 }
 
 }  // namespace dem

@@ -232,7 +232,7 @@ struct dem_scene {
   double *p3d_part = nullptr;   // kServoBlocks x 9 doubles
   P3d p3d_h{};
   bool p3d_on = false;
-  int *deg_ws = nullptr;       // 2 x kDegreeBuckets ints (integration order)
+  int *flip_max = nullptr;     // one int: largest shift a cell flip would make
   // launch shapes of the step kernels (none changes a result)
   int contact_block = 256, contact_per_sm = 8, integrate_block = 256, degree_order = 1;
   int step_graphs = -1;          // replay captured batches: 1 yes, 0 no, -1 small scenes
@@ -1076,7 +1076,7 @@ dem_status dem_scene_create(const dem_scene_desc *desc, dem_scene **out) {
   }
   if (dalloc(s, &s->mats_d, kMaxMat) || dalloc(s, &s->ds_d, 1) ||
       dalloc(s, &s->partials, 1024 * 32) || dalloc(s, &s->servo, kServoBlocks * 6) ||
-      dalloc(s, &s->deg_ws, 2 * kDegreeBuckets) || dalloc(s, &s->step_d, 1) || ensure_subs(s, 1)) {
+      dalloc(s, &s->flip_max, 1) || dalloc(s, &s->step_d, 1) || ensure_subs(s, 1)) {
     g_create_error = s->err;
     dem_scene_destroy(s);
     return DEM_ERR_OOM;
@@ -1132,7 +1132,7 @@ void dem_scene_destroy(dem_scene *s) {
   dfree(s, s->key); dfree(s, s->gF); dfree(s, s->gT); dfree(s, s->wpos); dfree(s, s->cinfo);
   dfree(s, s->cand_list); dfree(s, s->spill);
   dfree(s, s->cell_count); dfree(s, s->cell_start);
-  dfree(s, s->scan_ws); dfree(s, s->partials); dfree(s, s->servo); dfree(s, s->p3d_d); dfree(s, s->p3d_part); dfree(s, s->deg_ws);
+  dfree(s, s->scan_ws); dfree(s, s->partials); dfree(s, s->servo); dfree(s, s->p3d_d); dfree(s, s->p3d_part); dfree(s, s->flip_max);
   dfree(s, s->mats_d); dfree(s, s->cs_d); dfree(s, s->ds_d);
   dfree(s, s->grids_d); dfree(s, s->id_shift_d); dfree(s, s->bbox_keys); dfree(s, s->dt_keys);
   if (s->st) cudaStreamSynchronize(s->st);
@@ -2046,8 +2046,8 @@ dem_status stats_of(dem_scene *s, int q, dem_stats *o) {
   const bool have_table = s->table_fresh;
   const int nb = stats_blocks(nb_), nr = have_table ? stats_blocks(8 * nb_) : 0;
   const size_t words = 5 * (size_t)nb + 11 * (size_t)nr + (nr ? 1 : 0);
-  launch_stats(s->cur, s->tab[s->tc], s->mats_d, s->cs_d, scene_const(s), s->cap, b0, nb_, have_table,
-               s->mixed, nb, nr, s->partials, s->st);
+  launch_stats(s->cur, s->tab[s->tc], scene_const(s), s->cap, b0, nb_, have_table, s->mixed, nb, nr,
+               s->partials, s->st);
   CK(cudaGetLastError());
   CK(cudaMemcpyAsync(s->partials_h, s->partials, sizeof(double) * words, cudaMemcpyDeviceToHost, s->st));
   if ((r = wait(s))) return r;
@@ -2366,7 +2366,7 @@ dem_status dem_flip_cell(dem_scene *s, int sub, const int *flip, int *applied) {
     const Table &t = s->tab[s->tc];
     if (t.P > 0 && t.row_start != nullptr && s->N > 0) {
       const int multi = s->nsub() > 1;
-      int *maxabs = s->deg_ws;
+      int *maxabs = s->flip_max;
       CK(cudaMemsetAsync(maxabs, 0, sizeof(int), s->st));
       launch_flip_shift(t, s->cur.sid, multi, sub, Mi, maxabs, 0, s->st);
       int worst = 0;
