@@ -1790,7 +1790,8 @@ dem_status count_contacts(dem_scene *s, const int **off, long long *total) {
   if ((r = sync_host(s))) return r;
   const long long N = s->N;
   if (N == 0 || !s->table_fresh) return DEM_OK;
-  // 32 ints a body, at least 1024 bodies: counts (7 N), their sums (7 N + 1), scan workspace
+  // 32 ints a body, at least 1024 bodies: counts (7 N), their sums (7 N + 1), scan workspace (well
+  // under 2 N); the last 14 are free for records
   int *buf = reinterpret_cast<int *>(s->cand_list);
   const long long runs = s->has_walls ? 7 * N : N;
   int *cnt = buf, *sum = buf + 8 * s->cap, *ws = buf + 16 * s->cap;
@@ -1826,15 +1827,15 @@ dem_status dem_get_contacts(dem_scene *s, long long cap, long long *count, int *
   if (r) return r;
   if (count) *count = total;
   const long long m = std::min<long long>(cap, total);
-  // records go through a device buffer a chunk at a time (148 bytes a contact), smaller
-  // where the memory left does not hold the usual chunk
+  // records (148 bytes a contact) go through a device buffer, a chunk at a time: the rest of
+  // the list buffer where that holds them all or no other memory is to be had, else memory
+  // of its own
+  const long long rec = 3 * 8 * 5 + 8 + 4 + 4 + 12, spare = 14 * s->cap * (long long)sizeof(int) / rec;
   long long chunk = std::min<long long>(m, 1LL << 20);
-  char *buf = nullptr;
-  const long long rec = 3 * 8 * 5 + 8 + 4 + 4 + 12;
-  while (m > 0 && !buf) {
-    r = dalloc(s, &buf, chunk * rec);
-    if (r && chunk <= 1024) return r;
-    if (r) chunk = std::max<long long>(chunk / 8, 1024);
+  char *own = nullptr, *buf = reinterpret_cast<char *>(s->cand_list + 18 * s->cap);
+  if (chunk > spare) {
+    if (dalloc(s, &own, chunk * rec)) chunk = spare;
+    else buf = own;
   }
   for (long long at = 0; at < m && !r; at += chunk) {
     const long long k = std::min(chunk, m - at);
@@ -1869,7 +1870,7 @@ dem_status dem_get_contacts(dem_scene *s, long long cap, long long *count, int *
                             cudaMemcpyDeviceToHost, s->st);
     r = e == cudaSuccess ? wait(s) : cuda_fail(s, e, "contact export");
   }
-  dfree(s, buf);
+  dfree(s, own);
   return r;
 }
 
