@@ -210,6 +210,11 @@ __global__ void k_reorder(Bodies src, Bodies dst, long long N, long long cap,
   dst.wnear[p] = near;
 }
 
+__global__ void k_slots(const int *__restrict__ id, long long N, int *slot_of_id) {
+  const long long s = (long long)blockIdx.x * kT + threadIdx.x;
+  if (s < N) slot_of_id[id[s]] = (int)s;
+}
+
 // Does the shift of j seen from s leave the range of a packed shift?
 __device__ inline bool shift_overflow(const CellRec &cr, int s, int j, int code) {
   int w[3];
@@ -694,6 +699,10 @@ void launch_reorder(const Bodies &src, const Bodies &dst, long long N, long long
   if (N > 0)
     k_reorder<<<blocks(N), kT, 0, st>>>(src, dst, N, cap, tmp, key, start, raw, cr,
                                         new_to_old, slot_of_id, has_walls, mixed, id_shift, cs, multi);
+}
+
+void launch_slots(const int *id, long long N, int *slot_of_id, cudaStream_t st) {
+  if (N > 0) k_slots<<<blocks(N), kT, 0, st>>>(id, N, slot_of_id);
 }
 
 void launch_partners(CellRec cr, const int *sid, const int *id, long long N, const Grid *grids,

@@ -284,6 +284,8 @@ void launch_reorder(const Bodies &src, const Bodies &dst, long long N, long long
                     const int *tmp, const uint32_t *key, const int *start, CellRec raw, CellRec cr,
                     int *new_to_old, int *slot_of_id, int has_walls, int mixed,
                     const int *id_shift, const CellState *cs, int multi, cudaStream_t st);
+// slot_of_id of bodies in slot order
+void launch_slots(const int *id, long long N, int *slot_of_id, cudaStream_t st);
 // per-sub-scene bounding boxes as ordered keys (see collider.cu); keys preset
 void launch_bbox_sub(const Bodies &b, long long N, int cap, unsigned long long *keys, int nsm,
                      cudaStream_t st);

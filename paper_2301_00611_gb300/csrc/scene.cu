@@ -398,6 +398,7 @@ dem_status ensure_table(dem_scene *s, Table &t, long long rows, long long nbody)
     long long P = t.P;
     long long nc = std::max<long long>(rows + rows / 4, 1024);
     free_rows(s, t);
+    t.cap = t.P = 0;   // (until every array is there)
     if ((r = dalloc(s, &t.pair, nc)) || (r = dalloc(s, &t.cpack, nc)) ||
         (r = dalloc(s, &t.hfs, nc)) || (r = dalloc(s, &t.down, nc)) ||
         (r = dalloc(s, &t.found, nc)) || (r = dalloc(s, &t.bits, nc / 32 + 2)))
@@ -416,6 +417,7 @@ dem_status ensure_table(dem_scene *s, Table &t, long long rows, long long nbody)
   if (nbody + 1 > t.nbody_cap) {
     long long nb = std::max<long long>(nbody + 1, 64);
     dfree(s, t.row_start); dfree(s, t.down_start); dfree(s, t.ord);
+    t.nbody_cap = 0;
     if ((r = dalloc(s, &t.row_start, nb)) || (r = dalloc(s, &t.down_start, nb)) ||
         (r = dalloc(s, &t.ord, nb)))
       return r;
@@ -812,10 +814,18 @@ dem_status rebuild_core(dem_scene *s) {
   std::swap(s->cur, s->alt);
   s->N = n_live;
   const long long NL = n_live;
+  // A run that ends in an error puts the old order back: the last table goes by its slots, and
+  // a later run (after the cause is gone) takes the contact histories from there.
+  auto undo = [&](dem_status code) {
+    std::swap(s->cur, s->alt);
+    s->N = N;
+    launch_slots(s->cur.id, N, s->slot_of_id, s->st);
+    return code;
+  };
   // 4: partners of every body, prefix sums of the two counts
   Table &ot = s->tab[s->tc];
   Table &nt = s->tab[1 - s->tc];
-  if ((r = ensure_table(s, nt, 0, NL))) return r;
+  if ((r = ensure_table(s, nt, 0, NL))) return undo(r);
   // slots are packed in 26 bits of a list entry
   CandList cl{s->cand_list, s->cap < (1LL << 26) ? kCandKeep : 0, s->spill, s->spill_cap,
               reinterpret_cast<int *>(s->key), partners_many(NL)};
@@ -840,15 +850,17 @@ dem_status rebuild_core(dem_scene *s) {
   CK(cudaMemcpyAsync(&s->rb_h->totals[1], nt.down_start + NL, sizeof(int), cudaMemcpyDeviceToHost, s->st));
   CK(cudaMemcpyAsync(&s->rb_h->ds, s->ds_d, sizeof(DevStatus), cudaMemcpyDeviceToHost, s->st));
   if ((r = wait(s))) return r;
-  if (s->rb_h->ds.error) return status_error(s, s->rb_h->ds.error);
+  if (s->rb_h->ds.error) return undo(status_error(s, s->rb_h->ds.error));
   const long long P = s->rb_h->totals[0];
   // the number of pairs beyond 32 bits (see partners_many)
   const unsigned long long many = s->rb_h->ds.many_total, half = many / 2;
   const unsigned long long pairs = half + (unsigned)((unsigned)P - (unsigned)half);
   if (pairs > 0x7fffffffULL)
-    return fail(s, DEM_ERR_CAPACITY, "more than 2^31-1 candidate pairs (sweep margin or overlaps too large)");
-  if (P != s->rb_h->totals[1]) return fail(s, DEM_ERR_STATE, "internal: candidate count mismatch");
-  if ((r = ensure_table(s, nt, P, NL))) return r;
+    return undo(fail(s, DEM_ERR_CAPACITY,
+                     "more than 2^31-1 candidate pairs (sweep margin or overlaps too large)"));
+  if (P != s->rb_h->totals[1])
+    return undo(fail(s, DEM_ERR_STATE, "internal: candidate count mismatch"));
+  if ((r = ensure_table(s, nt, P, NL))) return undo(r);
   nt.P = P;
   // long lists that had no room: once more with a larger buffer (without the memory for it,
   // the row passes walk again for them)
@@ -1934,6 +1946,9 @@ dem_status dem_set_contacts(dem_scene *s, long long n, const int *id1, const int
   });
   const long long P = (long long)rows.size();
   Table &t = s->tab[s->tc];
+  s->table_fresh = false;   // from here on, whatever comes of it, the table is not the step's
+  s->need_rebuild = true;
+  s->check_lost = false;
   if ((r = ensure_table(s, t, std::max<long long>(P, 1), N))) return r;
   std::vector<int2> pair(P);
   std::vector<int> cp(P), rs(N + 1, 0);
@@ -1974,14 +1989,11 @@ dem_status dem_set_contacts(dem_scene *s, long long n, const int *id1, const int
   CK(cudaMemsetAsync(t.bits, 0xff, sizeof(unsigned) * (P / 32 + 2), s->st));   // all are real
   t.P = P;
   s->tab_nbody[s->tc] = N;
-  s->table_fresh = false;
   if (N > 0) CK(cudaMemcpyAsync(s->cur.flags, flags.data(), N, cudaMemcpyHostToDevice, s->st));
   if (s->has_walls)
     for (int w = 0; w < 6; ++w)
       CK(cudaMemcpyAsync(s->cur.whist + w * s->cap, wh.data() + w * N, sizeof(double4_32a) * N,
                          cudaMemcpyHostToDevice, s->st));
-  s->need_rebuild = true;
-  s->check_lost = false;
   return wait(s);
 }
 
