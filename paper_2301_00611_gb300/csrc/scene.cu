@@ -607,7 +607,8 @@ dem_status status_error(dem_scene *s, int e) {
 dem_status rebuild_core(dem_scene *s);
 
 // kernels the collider launches: bin, scan x2, scatter, reorder, partners, scan x2, rows,
-// downs, degree order, lost (small scans take one launch; a bounding box one more)
+// downs, degree order, lost (small scans take one launch; a bounding box and, in large scenes,
+// the long partner lists one more)
 dem_status rebuild(dem_scene *s) {
   if (s->timing) CK(cudaEventRecord(s->tev[0], s->st));
   dem_status r = rebuild_core(s);
